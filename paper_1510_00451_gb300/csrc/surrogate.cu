@@ -2,8 +2,8 @@
 // plain patch solve stays its fallback and the reference for its error).
 //
 // Features: per patch, the 17 x 17 low-mode DFT of the patch's band psi (patch
-// mean removed) times MLSD_SUR_PSI_SCALE / (tr(B)/2), then B/kappa, log kappa
-// (k_features), and the perturbation moments T_2..T_6 of the steady corrector
+// mean removed) times MLSD_SUR_PSI_SCALE / (tr(B)/2), then B/kappa, log kappa,
+// and the perturbation moments T_2..T_6 of the steady corrector
 // equation with the [2/2], [3/3], [4/4] Pade approximants of its resummed
 // series (from T_2..T_19), each as asinh(MLSD_SUR_T_SCALE x / tr B) (k_series):
 // 606 values stored as one bfloat16 row of MLSD_SUR_IN (640, zero padded).
@@ -28,85 +28,449 @@ constexpr int KMODE = 8;                   // local modes -8..8
 constexpr int NMODE = 2 * KMODE + 1;       // 17
 
 // ---------------------------------------------------------------------------
-// Features 0..581 and the zero padding: one CTA per patch.  The features of an
-// n x n patch are those of its nf x nf samples every sub-th node (nf = n / sub
-// <= 64: the samples are staged in shared memory)
-__global__ void k_features(const float *band, long long Nl, long long tile, int n, int sub,
-                           int n_macro, const int *pidx, long long count, const double *B,
-                           double kappa, __nv_bfloat16 *X, float *F32)
+// Features of a patch, and the perturbation moments behind features 582..605
+// and the baseline E of the network's target.  The features of an n x n patch
+// are those of its N x N samples every sub-th node (N = n / sub <= 64).
+// In index units (h = 1; the moments do not depend on h):
+//   v1 = -(psi[b+1][a] - psi[b-1][a]) / 2,  v2 = (psi[b][a+1] - psi[b][a-1]) / 2,
+//   g(k) = 1 / D(k), D = B11 (2 - 2 cos t1) + B22 (2 - 2 cos t2) + 2 B12 sin t1 sin t2,
+//   g(0) = 0 (-L0^{-1} is multiplication of the DFT by g),
+//   c_j^0 = -L0^{-1} v_j,  c_j^m = -L0^{-1} (v1 D0x + v2 D0y) c_j^{m-1},
+//   T_m = sym <v_i c_j^{m-2}>  (m = 2..19; means over the cells summed in FP32
+//   per thread and per warp, in FP64 over 8 partials).
+// Both fields go through one complex FFT as c1 + i c2: g is real and even in
+// k, so multiplying the transform of (f1 + i f2) by g transforms each part.
+// The first transform is that of psi itself, whose low modes are the window of
+// features 0..577.
+//
+// Layout: H threads a line, H N threads a patch (one warp a patch at N = 32, H = 1;
+// 128 threads at N = 64, H = 2).  A thread transforms N / H of its line's values in
+// registers (radix-2, decimation in time, twiddles as immediates); with H = 2 the last
+// stage goes to its partner by shuffles (lane ^ 16).  A pass reads lines of the
+// shared-memory field T and writes its results back as columns, so that the next pass
+// reads the other direction the same way: every read and write of T is conflict free
+// (line stride N + 1 complex values) and the same code serves rows and columns.  With
+// H = 2 the threads (col, 0) and (col, 1) keep the rows of the final column whose index
+// mod G is below and above G / 2 (runs of G / 2 rows): with G = 256 / N every FP32 chain
+// of the moment sums (rows of one residue mod G in a column) stays in one thread.
+//
+// What bounds it: at N = 32 FP32 issue and shared-memory transactions (four transposes of
+// the field a moment) about equally, 12 warps an SM; at N = 64 latency, 12 warps an SM where
+// shared memory holds three patches (one thread a line left 6 warps and missed the
+// instruction cache: 2.99 ms below instead of 2.09; two threads a line at N = 32 cost 2.28 ms
+// instead of 2.02).  One CTA of 256 threads a patch with the field in shared memory through
+// every radix-2 stage and a kernel of its own for the window took 8.48 ms for a surrogate
+// chain of two levels of 9216 patches of 32^2, now 2.02; and 8.00 ms for the features of
+// 4096 patches of 64^2, now 2.09.  The additions and products of a moment, and their order,
+// are those of that form: T_2..T_19 come out the same to the bit.
+constexpr int SERIES_M = 19;               // moments T_2..T_19
+
+// cos(2 pi k / 32)
+__host__ __device__ constexpr float cos32(int k)
 {
-    const int nf = n / sub;
+    constexpr float c[9] = {1.f, 0.980785251f, 0.923879504f, 0.831469595f, 0.707106769f,
+                            0.555570245f, 0.382683426f, 0.195090324f, 0.f};
+    k &= 31;
+    if (k > 16) k = 32 - k;
+    return k <= 8 ? c[k] : -c[16 - k];
+}
+
+// w b with w = (wx, -+ wy) (INV: +)
+template <bool INV>
+__device__ __forceinline__ float2 twiddle_mul(float2 b, float wx, float wy)
+{
+    if (INV) return make_float2(fmaf(b.x, wx, -__fmul_rn(b.y, wy)), fmaf(b.y, wx, __fmul_rn(b.x, wy)));
+    return make_float2(fmaf(b.x, wx, __fmul_rn(b.y, wy)), fmaf(-b.x, wy, __fmul_rn(b.y, wx)));
+}
+
+// radix-2 decimation in time over the M <= 32 values r (in bit-reversed order on entry),
+// stages HALF .. M / 2, twiddles e^{-+ 2 pi i k / M} (INV: +)
+template <int M, int HALF, bool INV>
+__device__ __forceinline__ void line_stage(float2 (&r)[M])
+{
+#pragma unroll
+    for (int j = 0; j < M / 2; ++j) {
+        const int pos = j & (HALF - 1), i0 = (j / HALF) * 2 * HALF + pos, i1 = i0 + HALF;
+        const int k = pos * (32 / (2 * HALF));
+        const float2 a = r[i0], b = r[i1];
+        float2 bw;
+        if (k == 0) bw = b;
+        else if (k == 8) bw = INV ? make_float2(-b.y, b.x) : make_float2(b.y, -b.x);
+        else bw = twiddle_mul<INV>(b, cos32(k), cos32(k + 24));
+        r[i0] = make_float2(__fadd_rn(a.x, bw.x), __fadd_rn(a.y, bw.y));
+        r[i1] = make_float2(__fsub_rn(a.x, bw.x), __fsub_rn(a.y, bw.y));
+    }
+    if constexpr (2 * HALF < M) line_stage<M, 2 * HALF, INV>(r);
+}
+
+__host__ __device__ constexpr int bit_reverse(int i, int n)
+{
+    int r = 0;
+    for (int m = 1; m < n; m <<= 1) r = 2 * r + ((i & m) ? 1 : 0);
+    return r;
+}
+
+template <int N>
+struct Series {
+    static constexpr int H = N == 32 ? 1 : 2;             // threads a line
+    static constexpr int NT = H * N, M = N / H;           // threads a patch, values a thread
+    static constexpr int P = N + 1;                       // line stride of T
+    static constexpr int G = 256 / N, RG = G / H;         // row groups of the sums, a thread's
+    static constexpr int MIN_CTAS = N == 32 ? 12 : 3;     // by shared memory
+    static constexpr int SP = N + 1;                      // stride of the sums' buffer
+    // float offsets
+    static constexpr int PSI = 2 * N * P, SYM = PSI + N * N, RED = SYM + (N / 2 + 1) * N;
+    static constexpr int CS = RED + (SERIES_M - 1) * 32;  // (1, 0) [N / 2], then cos, sin of 2 pi i / N [N]
+    static constexpr int SUM = CS + 3 * N, FLOATS = SUM + (H > 1 ? 4 * G * SP : 0);
+    static constexpr size_t BYTES = (size_t)FLOATS * 4;
+    static_assert(PSI % 2 == 0 && CS % 2 == 0 && SUM % 2 == 0, "8-byte alignment");
+
+    __device__ __forceinline__ static void sync()
+    {
+        if constexpr (NT == 32) __syncwarp();
+        else __syncthreads();
+    }
+    // grid row of value i of a thread (half h of its line) after a pass
+    __device__ __forceinline__ static int row(int i, int h)
+    {
+        if constexpr (H == 1) return i;
+        const int q = i % (M / 2);
+        return (i < M / 2 ? 0 : M) + G * (q / RG) + q % RG + RG * h;
+    }
+
+    // line `col` of T, transformed, into r: rows row(i, h); T may be rewritten afterwards
+    template <bool INV>
+    __device__ __forceinline__ static void pass(const float2 *T, const float2 *cs, float2 (&r)[M],
+                                                int col, int h)
+    {
+        if constexpr (H == 1) {
+#pragma unroll
+            for (int i = 0; i < M; ++i) r[i] = T[col * P + bit_reverse(i, M)];
+            sync();
+            line_stage<M, 1, INV>(r);
+        } else {
+            float2 y[M];
+#pragma unroll
+            for (int i = 0; i < M; ++i) y[i] = T[col * P + 2 * bit_reverse(i, M) + h];
+            sync();
+            line_stage<M, 1, INV>(y);
+            // last stage: (col, 0) holds a, (col, 1) b; w b there, then a + w b and a - w b
+            const float2 *tw = cs + (h ? M : 0);
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                const float2 w = tw[i];
+                y[i] = twiddle_mul<INV>(y[i], w.x, w.y);
+            }
+            const float sign = h ? -1.f : 1.f;
+#pragma unroll
+            for (int i = 0; i < M / 2; ++i) {
+                const int j0 = G * (i / RG) + i % RG, j1 = j0 + RG;
+                const float2 send = h ? y[j0] : y[j1], keep = h ? y[j1] : y[j0];
+                const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, send.x, 16),
+                                               __shfl_xor_sync(0xffffffffu, send.y, 16));
+                r[i] = make_float2(__fadd_rn(keep.x, got.x), __fadd_rn(keep.y, got.y));
+                r[i + M / 2] = make_float2(__fmul_rn(sign, __fsub_rn(keep.x, got.x)),
+                                           __fmul_rn(sign, __fsub_rn(keep.y, got.y)));
+            }
+        }
+    }
+    __device__ __forceinline__ static void store(float2 *T, const float2 (&r)[M], int col, int h)
+    {
+#pragma unroll
+        for (int i = 0; i < M; ++i) T[row(i, h) * P + col] = r[i];
+        sync();
+    }
+    // forward or inverse transform of T: rows, then columns
+    template <bool INV>
+    __device__ __forceinline__ static void transform(float2 *T, const float2 *cs, float2 (&r)[M],
+                                                     int col, int h)
+    {
+#pragma unroll 1
+        for (int k = 0; k < 2; ++k) {
+            pass<INV>(T, cs, r, col, h);
+            if (k == 0) store(T, r, col, h);
+        }
+    }
+};
+
+// sum of v[0..31] by the xor tree of a warp holding one value a lane
+template <typename T>
+__device__ __forceinline__ T tree32(const T *v)
+{
+    T s[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) s[c] = v[c] + v[c + 16];
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+        for (int c = 0; c < o; ++c) s[c] += s[c + o];
+    return s[0];
+}
+
+// One level of a transposing warp reduction: COUNT values a lane become COUNT / 2, lanes
+// with bit o set keeping the upper half; the pairs added are those of the xor tree.
+template <int COUNT>
+__device__ __forceinline__ void halve(float *v, int o, int lane)
+{
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < COUNT / 2; ++i) {
+        const float send = up ? v[i] : v[i + COUNT / 2], keep = up ? v[i + COUNT / 2] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+}
+
+template <int N>
+__global__ void __launch_bounds__(Series<N>::NT, Series<N>::MIN_CTAS)
+k_series(const float *band, long long Nl, long long tile, int n, int sub, int n_macro,
+         const int *pidx, long long count, const double *B, double kappa, __nv_bfloat16 *X,
+         float *F32, double *Eout)
+{
+    using S = Series<N>;
+    constexpr int P = S::P, H = S::H, RG = S::RG, M = S::M, SP = S::SP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float *psi = reinterpret_cast<float *>(smem_raw);              // [nf][nf]
-    float2 *Fr = reinterpret_cast<float2 *>(psi + nf * nf);        // [nf][17] row transforms
-    __shared__ double red[32];
-    __shared__ float2 tw[64];                                      // e^{-2 pi i r / nf}
+    float *sm = reinterpret_cast<float *>(smem_raw);
+    float2 *T = reinterpret_cast<float2 *>(sm);                      // [N][P] complex field
+    float *psi = sm + S::PSI;                                        // [N][N]
+    float *sym = sm + S::SYM;                                        // [N/2 + 1][N]: 1 / D(k)
+    float *red = sm + S::RED;                                        // [moment][8][4]
+    float2 *cs = reinterpret_cast<float2 *>(sm + S::CS);             // twiddles of the last stage
+    float *sums = sm + S::SUM;                                       // [G][4][SP]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int h = S::H == 1 ? 0 : lane >> 4, col = S::H == 1 ? (int)threadIdx.x : 16 * warp + (lane & 15);
     const long long item = blockIdx.x;
     if (item >= count) return;
     const long long p = pidx ? (long long)pidx[item] : item;
-    const long long ox = patch_origin(p % n_macro, n_macro, Nl, n);
-    const long long oy = patch_origin(p / n_macro, n_macro, Nl, n);
-    double sum = 0.0;
-    for (int c = threadIdx.x; c < nf * nf; c += blockDim.x) {
-        const int b = c / nf, a = c % nf;
-        const float v = patch_band(band, Nl, tile, p, ox, oy, n, a * sub, b * sub);
-        psi[c] = v;
-        sum += v;
-    }
-    for (int r = threadIdx.x; r < nf; r += blockDim.x) {
-        float s, c;
-        sincospif(-2.0f * (float)r / (float)nf, &s, &c);
-        tw[r] = make_float2(c, s);
-    }
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
-    __syncthreads();
-    double tot = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-    const float mean = (float)(tot / ((double)nf * nf));
-    // rows: Fr[b][k1] = sum_a (psi - mean) e^{-2 pi i k1 a / nf}
-    for (int t = threadIdx.x; t < nf * NMODE; t += blockDim.x) {
-        const int b = t / NMODE, k1 = t % NMODE - KMODE;
-        float sr = 0.f, si = 0.f;
-        const int step = (int)pmod_ll((long long)k1, nf);
-        int r = 0;
-        for (int a = 0; a < nf; ++a) {
-            const float2 w = tw[r];
-            const float v = psi[b * nf + a] - mean;
-            sr = fmaf(v, w.x, sr);
-            si = fmaf(v, w.y, si);
-            r += step;
-            if (r >= nf) r -= nf;
-        }
-        Fr[t] = make_float2(sr, si);
-    }
-    __syncthreads();
     const double B11 = B[3 * p], B12 = B[3 * p + 1], B22 = B[3 * p + 2];
-    const double trh = 0.5 * (B11 + B22);
-    const float scale = (float)(MLSD_SUR_PSI_SCALE / ((double)nf * nf * trh));
     __nv_bfloat16 *xr = X + item * (long long)MLSD_SUR_IN;
     float *fr = F32 ? F32 + item * (long long)MLSD_SUR_FEATURES : nullptr;
-    for (int t = threadIdx.x; t < NMODE * NMODE; t += blockDim.x) {
-        const int k2 = t / NMODE - KMODE, k1i = t % NMODE;
-        float sr = 0.f, si = 0.f;
-        const int step = (int)pmod_ll((long long)k2, nf);
-        int r = 0;
-        for (int b = 0; b < nf; ++b) {
-            const float c = tw[r].x, s = tw[r].y;
-            r += step;
-            if (r >= nf) r -= nf;
-            const float2 f = Fr[b * NMODE + k1i];
-            // (f.x + i f.y)(c + i s)
-            sr += f.x * c - f.y * s;
-            si += f.x * s + f.y * c;
+
+    // ---- the patch's samples and their mean in FP64 ----
+    float s1, co1;
+    sincospif(2.0f * (float)col / (float)N, &s1, &co1);
+    if (h == 0) cs[N / 2 + col] = make_float2(co1, s1);
+    else if (col < N / 2) cs[col] = make_float2(1.f, 0.f);
+    float mean;
+    {
+        double acc[RG];
+#pragma unroll
+        for (int q = 0; q < RG; ++q) acc[q] = 0.0;
+        const float *src;
+        long long y0 = 0, ld, wrap = 0;
+        if (tile) {
+            src = band + p * tile + (long long)col * sub;
+            ld = n;
+        } else {
+            // the patch is at most one band grid wide: one wrap at most
+            src = band + pmod_ll(patch_origin(p % n_macro, n_macro, Nl, n) + (long long)col * sub, Nl);
+            y0 = pmod_ll(patch_origin(p / n_macro, n_macro, Nl, n), Nl);
+            ld = wrap = Nl;
         }
-        const float re = sr * scale, im = si * scale;
-        xr[2 * t] = __float2bfloat16_rn(re);
-        xr[2 * t + 1] = __float2bfloat16_rn(im);
-        if (fr) { fr[2 * t] = re; fr[2 * t + 1] = im; }
+#pragma unroll 8
+        for (int i = 0; i < M; ++i) {
+            const int b = S::row(i, h);
+            long long y = y0 + (long long)b * sub;
+            if (wrap && y >= wrap) y -= wrap;
+            psi[b * N + col] = src[y * ld];
+        }
+#pragma unroll
+        for (int i = 0; i < M; ++i) acc[i % RG] += psi[S::row(i, h) * N + col];
+        double *part = reinterpret_cast<double *>(T);                // [G][SP]
+#pragma unroll
+        for (int q = 0; q < RG; ++q) part[(q + RG * h) * SP + col] = acc[q];
+        S::sync();
+        // partial w: row group w (N = 32), or group w / 2 and column half w % 2
+        double v = 0.0, tot = 0.0;
+        if (lane < 8) v = tree32(part + (N == 32 ? lane : lane >> 1) * SP + (N == 32 ? 0 : 32 * (lane & 1)));
+#pragma unroll
+        for (int w = 0; w < 8; ++w) tot += __shfl_sync(0xffffffffu, v, w);
+        mean = (float)(tot / (double)(N * N));
+        S::sync();                                                   // part is read
     }
-    const int t = 2 * NMODE * NMODE + threadIdx.x;
-    if (t < MLSD_SUR_IN && (t < 582 || t >= MLSD_SUR_FEATURES)) {   // 582..605: k_series
+    // ---- the symbol of -L0^{-1}: rows 0 .. N/2 (g is even in k) ----
+#pragma unroll 4
+    for (int b = h; b <= N / 2; b += H) {
+        const float co2 = cs[N / 2 + b].x, s2 = cs[N / 2 + b].y;
+        const float D = fmaf(__fmul_rn(2.f * (float)B12, s1), s2,
+                             fmaf((float)B11, fmaf(-2.f, co1, 2.f),
+                                  __fmul_rn((float)B22, fmaf(-2.f, co2, 2.f))));
+        sym[b * N + col] = (b == 0 && col == 0) ? 0.f : 1.f / D;
+    }
+
+    const int le = (col + 1) & (N - 1), lw = (col + N - 1) & (N - 1), lm = (N - col) & (N - 1);
+    const float inv = 1.0f / (float)(N * N);
+    float2 r[M];
+    // m = 1: transform of psi, giving the window and c^0; m >= 2: moment m from the
+    // iterate c^{m-2} (r: this thread's rows of its column, unscaled), then c^{m-1}
+    for (int m = 1; m <= SERIES_M; ++m) {
+        if (m == 1) {
+#pragma unroll
+            for (int i = 0; i < M; ++i) r[i] = make_float2(psi[S::row(i, h) * N + col] - mean, 0.f);
+        } else {
+#pragma unroll
+            for (int i = 0; i < M; ++i) r[i] = make_float2(__fmul_rn(r[i].x, inv), __fmul_rn(r[i].y, inv));
+            if constexpr (H > 1) S::store(T, r, col, h);
+            float acc[4 * RG];
+#pragma unroll
+            for (int q = 0; q < 4 * RG; ++q) acc[q] = 0.f;
+            float2 z[H > 1 ? M : 1];
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                const int b = S::row(i, h), bp = (b + 1) & (N - 1), bm = (b + N - 1) & (N - 1);
+                const float a1 = 0.5f * (psi[bm * N + col] - psi[bp * N + col]);
+                const float a2 = 0.5f * (psi[b * N + le] - psi[b * N + lw]);
+                // columns col +- 1: H = 1 from the neighbouring lanes, else from T; rows b +- 1:
+                // in this thread inside a run of RG rows, else in T
+                const float2 c = r[i];
+                float2 e, w, u, d;
+                if constexpr (H == 1) {
+                    e = make_float2(__shfl_sync(0xffffffffu, c.x, le), __shfl_sync(0xffffffffu, c.y, le));
+                    w = make_float2(__shfl_sync(0xffffffffu, c.x, lw), __shfl_sync(0xffffffffu, c.y, lw));
+                    u = r[(i + 1) % M];
+                    d = r[(i + M - 1) % M];
+                } else {
+                    e = T[b * P + le];
+                    w = T[b * P + lw];
+                    u = i % RG < RG - 1 ? r[(i + 1) % M] : T[bp * P + col];
+                    d = i % RG > 0 ? r[(i + M - 1) % M] : T[bm * P + col];
+                }
+                float *s = acc + 4 * (i % RG);
+                s[0] = fmaf(a1, c.x, s[0]);
+                s[1] = fmaf(a1, c.y, s[1]);
+                s[2] = fmaf(a2, c.x, s[2]);
+                s[3] = fmaf(a2, c.y, s[3]);
+                const float d1x = 0.5f * (e.x - w.x), d1y = 0.5f * (u.x - d.x);
+                const float d2x = 0.5f * (e.y - w.y), d2y = 0.5f * (u.y - d.y);
+                const float2 f = make_float2(fmaf(a1, d1x, __fmul_rn(a2, d1y)),
+                                             fmaf(a1, d2x, __fmul_rn(a2, d2y)));
+                if constexpr (H == 1) T[b * P + col] = f;
+                else z[i] = f;
+            }
+            // partial sum w (rows of one group over 32 columns, as the mean's), quantity q, in
+            // lane 4 w + q
+            if constexpr (H == 1) {
+                halve<32>(acc, 16, lane); halve<16>(acc, 8, lane); halve<8>(acc, 4, lane);
+                halve<4>(acc, 2, lane); halve<2>(acc, 1, lane);
+                red[(m - 2) * 32 + lane] = acc[0];
+            } else {
+#pragma unroll
+                for (int q = 0; q < 4 * RG; ++q) sums[(q + 4 * RG * h) * SP + col] = acc[q];
+                __syncthreads();
+                if (warp == 0)
+                    red[(m - 2) * 32 + lane] =
+                        tree32(sums + (4 * (lane >> 3) + (lane & 3)) * SP + 32 * ((lane >> 2) & 1));
+            }
+            if (m == SERIES_M) break;
+            if constexpr (H > 1) {
+#pragma unroll
+                for (int i = 0; i < M; ++i) r[i] = z[i];
+            }
+        }
+        if (H > 1 || m == 1) S::store(T, r, col, h);
+        else S::sync();
+        S::template transform<false>(T, cs, r, col, h);              // wavenumber k1 = col, r: k2
+        if (m == 1) {
+            if (col <= KMODE || col >= N - KMODE) {
+                const int k1i = col <= KMODE ? col + KMODE : col - N + KMODE;
+                const float scale = (float)(MLSD_SUR_PSI_SCALE / ((double)N * N * (0.5 * (B11 + B22))));
+#pragma unroll
+                for (int i = 0; i < M; ++i) {
+                    const int b = S::row(i, h), k2i = b <= KMODE ? b + KMODE : b - N + KMODE;
+                    if (k2i < 0) continue;                           // |k2| > KMODE
+                    const float re = r[i].x * scale, im = r[i].y * scale;
+                    const int t = k2i * NMODE + k1i;
+                    *reinterpret_cast<__nv_bfloat162 *>(xr + 2 * t) =
+                        __nv_bfloat162(__float2bfloat16_rn(re), __float2bfloat16_rn(im));
+                    if (fr) *reinterpret_cast<float2 *>(fr + 2 * t) = make_float2(re, im);
+                }
+            }
+            // c^0: transform of c1 + i c2 = g (-s1 - i s2) psihat
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                const float s2 = cs[N / 2 + S::row(i, h)].y;
+                r[i] = make_float2(fmaf(r[i].y, s2, -__fmul_rn(r[i].x, s1)),
+                                   fmaf(-r[i].x, s2, -__fmul_rn(r[i].y, s1)));
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            const int b = S::row(i, h);
+            const float gk = i <= M / 2 - (H - 1) ? sym[b * N + col] : sym[(N - b) * N + lm];
+            r[i] = make_float2(__fmul_rn(r[i].x, gk), __fmul_rn(r[i].y, gk));
+        }
+        S::store(T, r, col, h);
+        S::template transform<true>(T, cs, r, col, h);
+    }
+    if (warp > 0) return;
+    __syncwarp();
+    // ---- moments, resummation and features 578..639: one warp ----
+    // T_m (FP64) from the 8 partial sums of its four products, in their order
+    double *tm = reinterpret_cast<double *>(T);                      // [moment][4]
+    for (int i = lane; i < (SERIES_M - 1) * 4; i += 32) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += (double)red[(i >> 2) * 32 + 4 * w + (i & 3)];
+        tm[i] = t;
+    }
+    __syncwarp();
+    const double nn = (double)(N * N);
+    auto moment = [&](int m, int c) {                                // T_{m+2}, component c
+        return c == 0 ? tm[4 * m] / nn : c == 1 ? 0.5 * (tm[4 * m + 1] + tm[4 * m + 2]) / nn
+                                                : tm[4 * m + 3] / nn;
+    };
+    // Resummation: pairs p_k = T_(2k+2) + T_(2k+3), k = 0..8, and the [K/K] Pade
+    // approximants at 1 of sum_k p_k x^k, K = 2, 3, 4, by Wynn's epsilon algorithm on
+    // the partial sums, lane 9 c + j holding entry j of component c's current column.
+    // The tables of the smaller K are the first 2K + 1 entries of the largest; where a
+    // difference of a table vanishes, it keeps the last even column reached.
+    const int comp = min(lane / 9, 2), j = lane < 27 ? lane - 9 * comp : 8;
+    double cur = 0.0, prev = 0.0;
+    for (int k = 0; k < 9; ++k)
+        if (k <= j) cur += moment(2 * k, comp) + moment(2 * k + 1, comp);
+    double best[3];
+    bool live[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        best[q] = __shfl_sync(0xffffffffu, cur, 9 * comp + 2 * (q + 2));
+        live[q] = true;
+    }
+    for (int k = 1; k <= 8; ++k) {
+        const double d = __shfl_down_sync(0xffffffffu, cur, 1) - cur;
+        const double up = __shfl_down_sync(0xffffffffu, prev, 1);
+        const unsigned zero = __ballot_sync(0xffffffffu, fabs(d) < 1e-300) >> (9 * comp);
+        prev = cur;
+        cur = up + 1.0 / d;
+        const double first = __shfl_sync(0xffffffffu, cur, 9 * comp);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const int K2 = 2 * (q + 2);                              // this table's last column
+            if (k > K2) continue;
+            live[q] = live[q] && !(zero & ((1u << (K2 + 1 - k)) - 1u));
+            if (live[q] && !(k & 1)) best[q] = first;
+        }
+    }
+    const double sc = MLSD_SUR_T_SCALE / (B11 + B22);
+    {
+        const int c = lane % 3;
+        const double b2 = __shfl_sync(0xffffffffu, best[0], 9 * c), b3 = __shfl_sync(0xffffffffu, best[1], 9 * c);
+        const double b4 = __shfl_sync(0xffffffffu, best[2], 9 * c);
+        if (lane < 24) {
+            const double x = lane < 15 ? moment(lane / 3, c) : lane < 18 ? b2 : lane < 21 ? b3 : b4;
+            const float f = (float)asinh(sc * x);
+            xr[582 + lane] = __float2bfloat16_rn(f);
+            if (fr) fr[582 + lane] = f;
+        }
+    }
+    if (Eout) {
+        // E and how far it is from converged, max_c |[4/4]_c - [3/3]_c| (NaN if any is)
+        const double gc = fabs(best[2] - best[1]);
+        const double g0 = __shfl_sync(0xffffffffu, gc, 0), g1 = __shfl_sync(0xffffffffu, gc, 9),
+                     g2 = __shfl_sync(0xffffffffu, gc, 18);
+        if (lane < 27 && j == 0) Eout[item * 4 + comp] = best[2];
+        if (lane == 0)
+            Eout[item * 4 + 3] = (g0 == g0 && g1 == g1 && g2 == g2) ? fmax(g0, fmax(g1, g2)) : g0 + g1 + g2;
+    }
+    for (int t = 578 + lane; t < MLSD_SUR_IN; t += 32) {
+        if (t >= 582 && t < MLSD_SUR_FEATURES) continue;
         float v = 0.f;
         if (t == 578) v = (float)(B11 / kappa);
         else if (t == 579) v = (float)(B12 / kappa);
@@ -117,25 +481,7 @@ __global__ void k_features(const float *band, long long Nl, long long tile, int 
     }
 }
 
-// ---------------------------------------------------------------------------
-// Perturbation moments of the steady corrector equation (features 582..605 and
-// the baseline E of the network's target).  In index units (h = 1; the moments
-// do not depend on h):
-//   v1 = -(psi[b+1][a] - psi[b-1][a]) / 2,  v2 = (psi[b][a+1] - psi[b][a-1]) / 2,
-//   g(k) = 1 / D(k), D = B11 (2 - 2 cos t1) + B22 (2 - 2 cos t2) + 2 B12 sin t1 sin t2,
-//   g(0) = 0 (-L0^{-1} is multiplication of the DFT by g),
-//   c_j^0 = -L0^{-1} v_j,  c_j^m = -L0^{-1} (v1 D0x + v2 D0y) c_j^{m-1},
-//   T_m = sym <v_i c_j^{m-2}>  (m = 2..19; means over the cells summed in FP32
-//   per thread and per warp, in FP64 across the warps).
-// Both fields go through one complex FFT as c1 + i c2: g is real and even in
-// k, so multiplying the transform of (f1 + i f2) by g transforms each part.
-// One CTA of 256 threads per patch, everything in shared memory: the complex
-// work field, v1, v2, c1, c2, the symbol g and the twiddles (n = 32: 28 KB,
-// n = 64: 112 KB).  Radix-2 FFT along rows, then columns, in FP32.
-// Resummation (FP64, one thread per component): pairs p_k = T_(2k+2) + T_(2k+3),
-// k = 0..8, and the [K/K] Pade approximants at 1 of sum_k p_k x^k by Wynn's
-// epsilon algorithm on the partial sums (K = 2, 3, 4); E = [4/4] and
-// Eout[item] = (E11, E12, E22, max_c |[4/4]_c - [3/3]_c|).
+// Radix-2 FFT of a complex N x N field in shared memory, rows then columns (k_periodize)
 template <int N>
 __device__ void fft2_smem(float2 *z, const float2 *tw, bool inverse)
 {
@@ -171,200 +517,6 @@ __device__ void fft2_smem(float2 *z, const float2 *tw, bool inverse)
             }
             __syncthreads();
         }
-    }
-}
-
-// block sum of 4 doubles (256 threads = 8 warps); every thread gets the totals
-__device__ __forceinline__ void block_sum4(double (&v)[4], double (*red)[8])
-{
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
-    if ((threadIdx.x & 31) == 0)
-        for (int q = 0; q < 4; ++q) red[q][threadIdx.x >> 5] = v[q];
-    __syncthreads();
-    for (int q = 0; q < 4; ++q) {
-        double t = 0.0;
-        for (int w = 0; w < 8; ++w) t += red[q][w];
-        v[q] = t;
-    }
-    __syncthreads();
-}
-
-// block sum of 4 floats into 4 doubles held by thread 0 only: FP32 within a
-// thread and across the warp, FP64 for the 8 warp partials (the FP64 pipe of
-// this part is narrow, so the per-thread and per-warp sums stay in FP32)
-__device__ __forceinline__ void block_sum4_root(float (&v)[4], double (*red)[8], double (&out)[4])
-{
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
-    if ((threadIdx.x & 31) == 0)
-        for (int q = 0; q < 4; ++q) red[q][threadIdx.x >> 5] = (double)v[q];
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int q = 0; q < 4; ++q) {
-            double t = 0.0;
-            for (int w = 0; w < 8; ++w) t += red[q][w];
-            out[q] = t;
-        }
-}
-
-// [K/K] at 1 of sum_k c_k x^k by Wynn's epsilon algorithm on the partial sums
-// (c_0..c_2K, K <= 4); where a difference vanishes, the last even column reached
-__device__ double wynn_dev(const double *c, int K)
-{
-    double ea[10], eb[10];
-    double *prev = ea, *cur = eb;
-    const int n = 2 * K + 1;
-    double acc = 0.0;
-    for (int j = 0; j < n; ++j) { acc += c[j]; cur[j] = acc; prev[j] = 0.0; }
-    prev[n] = 0.0;
-    double best = cur[n - 1];
-    int len = n;
-    for (int k = 1; k <= 2 * K; ++k) {
-        for (int j = 0; j < len - 1; ++j) {          // in place: prev[j] <- eps_{k}^{(j)}
-            const double d = cur[j + 1] - cur[j];
-            if (fabs(d) < 1e-300) return best;
-            prev[j] = prev[j + 1] + 1.0 / d;
-        }
-        double *t = prev; prev = cur; cur = t;
-        len -= 1;
-        if ((k & 1) == 0) best = cur[0];
-    }
-    return cur[0];
-}
-
-constexpr int SERIES_M = 19;               // moments T_2..T_19
-
-template <int N>
-__global__ void __launch_bounds__(256) k_series(const float *band, long long Nl, long long tile,
-                                                int n, int sub, int n_macro, const int *pidx,
-                                                long long count, const double *B,
-                                                __nv_bfloat16 *X, float *F32, double *Eout)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2 *z = reinterpret_cast<float2 *>(smem_raw);               // [N][N] complex
-    float *v1 = reinterpret_cast<float *>(z + N * N);                // [N][N] each:
-    float *v2 = v1 + N * N, *c1 = v2 + N * N, *c2 = c1 + N * N;      // velocity, iterates,
-    float *g = c2 + N * N;                                           // 1 / D(k)
-    float2 *tw = reinterpret_cast<float2 *>(g + N * N);              // [N/2]
-    float *psi = c1;                                                 // psi until v is formed
-    __shared__ double red[4][8];
-    __shared__ double Tm[SERIES_M - 1][3];
-    const long long item = blockIdx.x;
-    if (item >= count) return;
-    const long long p = pidx ? (long long)pidx[item] : item;
-    const long long ox = patch_origin(p % n_macro, n_macro, Nl, n);
-    const long long oy = patch_origin(p / n_macro, n_macro, Nl, n);
-    const double B11 = B[3 * p], B12 = B[3 * p + 1], B22 = B[3 * p + 2];
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-        const int b = e / N, a = e % N;
-        const float v = patch_band(band, Nl, tile, p, ox, oy, n, a * sub, b * sub);
-        psi[e] = v;
-        acc[0] += v;
-        // the symbol of -L0^{-1}, once per patch
-        float s1, co1, s2, co2;
-        sincospif(2.0f * (float)a / (float)N, &s1, &co1);
-        sincospif(2.0f * (float)b / (float)N, &s2, &co2);
-        const float D = (float)B11 * (2.f - 2.f * co1) + (float)B22 * (2.f - 2.f * co2)
-                        + 2.f * (float)B12 * s1 * s2;
-        g[e] = e == 0 ? 0.f : 1.f / D;
-    }
-    for (int k = threadIdx.x; k < N / 2; k += blockDim.x) {
-        float sn, cs;
-        sincospif(-2.0f * (float)k / (float)N, &sn, &cs);
-        tw[k] = make_float2(cs, sn);
-    }
-    block_sum4(acc, red);
-    const float mean = (float)(acc[0] / (double)(N * N));
-    for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-        const int b = e / N, a = e % N;
-        const int ap = (a + 1) & (N - 1), am = (a + N - 1) & (N - 1);
-        const int bp = (b + 1) & (N - 1), bm = (b + N - 1) & (N - 1);
-        v1[e] = 0.5f * (psi[bm * N + a] - psi[bp * N + a]);
-        v2[e] = 0.5f * (psi[b * N + ap] - psi[b * N + am]);
-        z[e] = make_float2(psi[e] - mean, 0.f);
-    }
-    __syncthreads();
-    fft2_smem<N>(z, tw, false);
-    // c^0: transform of c1 + i c2 = g (-s1 - i s2) psihat
-    for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-        const int k1 = e % N, k2 = e / N;
-        const float s1 = sinpif(2.0f * (float)k1 / (float)N), s2 = sinpif(2.0f * (float)k2 / (float)N);
-        const float2 q = z[e];
-        z[e] = make_float2(g[e] * (-q.x * s1 + q.y * s2), g[e] * (-q.x * s2 - q.y * s1));
-    }
-    __syncthreads();
-    fft2_smem<N>(z, tw, true);
-    const float inv = 1.0f / (float)(N * N);
-    for (int e = threadIdx.x; e < N * N; e += blockDim.x) { c1[e] = z[e].x * inv; c2[e] = z[e].y * inv; }
-    __syncthreads();
-    for (int m = 2; m <= SERIES_M; ++m) {
-        float sm[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-            const float a1 = v1[e], a2 = v2[e];
-            sm[0] = fmaf(a1, c1[e], sm[0]); sm[1] = fmaf(a1, c2[e], sm[1]);
-            sm[2] = fmaf(a2, c1[e], sm[2]); sm[3] = fmaf(a2, c2[e], sm[3]);
-            if (m < SERIES_M) {
-                const int b = e / N, a = e % N;
-                const int ap = (a + 1) & (N - 1), am = (a + N - 1) & (N - 1);
-                const int bp = (b + 1) & (N - 1), bm = (b + N - 1) & (N - 1);
-                const float d1x = 0.5f * (c1[b * N + ap] - c1[b * N + am]);
-                const float d1y = 0.5f * (c1[bp * N + a] - c1[bm * N + a]);
-                const float d2x = 0.5f * (c2[b * N + ap] - c2[b * N + am]);
-                const float d2y = 0.5f * (c2[bp * N + a] - c2[bm * N + a]);
-                z[e] = make_float2(fmaf(a1, d1x, a2 * d1y), fmaf(a1, d2x, a2 * d2y));
-            }
-        }
-        double tot[4];
-        block_sum4_root(sm, red, tot);
-        if (threadIdx.x == 0) {
-            const double nn = (double)(N * N);
-            Tm[m - 2][0] = tot[0] / nn;
-            Tm[m - 2][1] = 0.5 * (tot[1] + tot[2]) / nn;
-            Tm[m - 2][2] = tot[3] / nn;
-        }
-        if (m == SERIES_M) break;
-        fft2_smem<N>(z, tw, false);
-        for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-            const float q = g[e];
-            z[e] = make_float2(z[e].x * q, z[e].y * q);
-        }
-        __syncthreads();
-        fft2_smem<N>(z, tw, true);
-        for (int e = threadIdx.x; e < N * N; e += blockDim.x) { c1[e] = z[e].x * inv; c2[e] = z[e].y * inv; }
-        __syncthreads();
-    }
-    __syncthreads();
-    const double sc = MLSD_SUR_T_SCALE / (B11 + B22);
-    __nv_bfloat16 *xr = X + item * (long long)MLSD_SUR_IN;
-    float *fr = F32 ? F32 + item * (long long)MLSD_SUR_FEATURES : nullptr;
-    if (threadIdx.x < 3) {
-        const int c = threadIdx.x;
-        double pk[9];
-        for (int k = 0; k < 9; ++k) pk[k] = Tm[2 * k][c] + Tm[2 * k + 1][c];
-        const double P2 = wynn_dev(pk, 2), P3 = wynn_dev(pk, 3), E = wynn_dev(pk, 4);
-        red[0][c] = fabs(E - P3);
-        if (Eout) Eout[item * 4 + c] = E;
-        const float f2 = (float)asinh(sc * P2), f3 = (float)asinh(sc * P3),
-                    fe = (float)asinh(sc * E);
-        xr[597 + c] = __float2bfloat16_rn(f2);
-        xr[600 + c] = __float2bfloat16_rn(f3);
-        xr[603 + c] = __float2bfloat16_rn(fe);
-        if (fr) { fr[597 + c] = f2; fr[600 + c] = f3; fr[603 + c] = fe; }
-    }
-    if (threadIdx.x < 15) {
-        const float f = (float)asinh(sc * Tm[threadIdx.x / 3][threadIdx.x % 3]);
-        xr[582 + threadIdx.x] = __float2bfloat16_rn(f);
-        if (fr) fr[582 + threadIdx.x] = f;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && Eout) {
-        const double g0 = fmax(red[0][0], fmax(red[0][1], red[0][2]));
-        Eout[item * 4 + 3] = (red[0][0] == red[0][0] && red[0][1] == red[0][1] &&
-                              red[0][2] == red[0][2]) ? g0 : red[0][0] + red[0][1] + red[0][2];
     }
 }
 
@@ -1032,15 +1184,16 @@ long long sur_param_count(int h)
 template <int N>
 static cudaError_t launch_series(const float *band, long long Nl, long long tile, int n, int sub,
                                  int n_macro, const int *pidx, long long count, const double *B,
-                                 void *X, float *F32, double *E, cudaStream_t s)
+                                 double kappa, void *X, float *F32, double *E, cudaStream_t s)
 {
-    const size_t smem = (size_t)N * N * (8 + 5 * 4) + (size_t)N / 2 * 8;
     cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&k_series<N>),
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)Series<N>::BYTES);
     if (e != cudaSuccess) return e;
     count_launches(1);
-    k_series<N><<<(unsigned)count, 256, smem, s>>>(band, Nl, tile, n, sub, n_macro, pidx, count,
-                                                   B, static_cast<__nv_bfloat16 *>(X), F32, E);
+    k_series<N><<<(unsigned)count, Series<N>::NT, Series<N>::BYTES, s>>>(band, Nl, tile, n, sub, n_macro, pidx,
+                                                            count, B, kappa,
+                                                            static_cast<__nv_bfloat16 *>(X), F32, E);
     return cudaGetLastError();
 }
 
@@ -1053,17 +1206,8 @@ cudaError_t launch_features(const float *band, long long Nl, long long tile, int
     if (count == 0) return cudaSuccess;
     if (n != 32 && n != 64 && n != 128 && n != 256) return cudaErrorInvalidValue;
     const int nf = n < 64 ? n : 64, sub = n / nf;
-    const size_t smem = (size_t)nf * nf * 4 + (size_t)nf * NMODE * 8;
-    cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&k_features),
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    count_launches(1);
-    k_features<<<(unsigned)count, 320, smem, s>>>(band, Nl, tile, n, sub, n_macro, pidx, count, B,
-                                                  kappa, static_cast<__nv_bfloat16 *>(X), F32);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return nf == 32 ? launch_series<32>(band, Nl, tile, n, sub, n_macro, pidx, count, B, X, F32, E, s)
-                    : launch_series<64>(band, Nl, tile, n, sub, n_macro, pidx, count, B, X, F32, E, s);
+    return nf == 32 ? launch_series<32>(band, Nl, tile, n, sub, n_macro, pidx, count, B, kappa, X, F32, E, s)
+                    : launch_series<64>(band, Nl, tile, n, sub, n_macro, pidx, count, B, kappa, X, F32, E, s);
 }
 
 template <int N>
