@@ -111,7 +111,8 @@ struct ModeGroups {
     const int *k2;           // [n_modes]
     const double *re, *im;   // [n_modes]
 };
-// G scratch: [n_groups][Nl] double2.  out: float or double [Nl][Nl].
+// G scratch: [n_groups + 1][Nl] double2 (the last row: the roots of unity).
+// out: float or double [Nl][Nl].
 cudaError_t launch_band_synth(const ModeGroups &m, long long Nl, double2 *G, void *out,
                               int out_double, cudaStream_t s);
 

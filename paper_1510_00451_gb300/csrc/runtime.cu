@@ -130,36 +130,80 @@ int level_of_mag(int m, int L, const double *e)
 
 struct HostMode { int k1, k2; double re, im; };
 
-// group modes by k1 and upload: returns device ModeGroups pointing into `blob`
-int upload_groups(mlsd_levels *h, const std::vector<HostMode> &modes, ModeGroups &g)
+// The mode list of a real field with every mode in the half plane k1 > 0, or k1 = 0 and
+// k2 >= 0 (a mode and its mirror with the conjugate coefficient have the same real part), equal
+// modes merged: half the modes and half the k1 groups to synthesise.  Sorted by (k1, k2).
+std::vector<HostMode> fold_modes(const std::vector<HostMode> &modes)
 {
     std::vector<HostMode> ms = modes;
-    std::sort(ms.begin(), ms.end(), [](const HostMode &a, const HostMode &b) {
+    for (HostMode &m : ms)
+        if (m.k1 < 0 || (m.k1 == 0 && m.k2 < 0)) m = {-m.k1, -m.k2, m.re, -m.im};
+    std::stable_sort(ms.begin(), ms.end(), [](const HostMode &a, const HostMode &b) {
         return a.k1 != b.k1 ? a.k1 < b.k1 : a.k2 < b.k2;
     });
-    std::vector<int> gk1, gofs, k2;
-    std::vector<double> re, im;
+    size_t n = 0;
     for (size_t t = 0; t < ms.size(); ++t) {
-        if (t == 0 || ms[t].k1 != ms[t - 1].k1) { gk1.push_back(ms[t].k1); gofs.push_back((int)t); }
-        k2.push_back(ms[t].k2); re.push_back(ms[t].re); im.push_back(ms[t].im);
+        if (n > 0 && ms[n - 1].k1 == ms[t].k1 && ms[n - 1].k2 == ms[t].k2) {
+            ms[n - 1].re += ms[t].re;
+            ms[n - 1].im += ms[t].im;
+        } else {
+            ms[n++] = ms[t];
+        }
     }
-    gofs.push_back((int)ms.size());
-    g.n_groups = (int)gk1.size();
-    if (ms.empty()) { g.gk1 = g.gofs = g.k2 = nullptr; g.re = g.im = nullptr; return MLSD_OK; }
-    void *p[5];
-    int rc;
-    if ((rc = dev_alloc(h, &p[0], gk1.size() * 4))) return rc;
-    if ((rc = dev_alloc(h, &p[1], gofs.size() * 4))) return rc;
-    if ((rc = dev_alloc(h, &p[2], k2.size() * 4))) return rc;
-    if ((rc = dev_alloc(h, &p[3], re.size() * 8))) return rc;
-    if ((rc = dev_alloc(h, &p[4], im.size() * 8))) return rc;
-    CK(cudaMemcpy(p[0], gk1.data(), gk1.size() * 4, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(p[1], gofs.data(), gofs.size() * 4, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(p[2], k2.data(), k2.size() * 4, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(p[3], re.data(), re.size() * 8, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(p[4], im.data(), im.size() * 8, cudaMemcpyHostToDevice));
-    g.gk1 = (int *)p[0]; g.gofs = (int *)p[1]; g.k2 = (int *)p[2];
-    g.re = (double *)p[3]; g.im = (double *)p[4];
+    ms.resize(n);
+    return ms;
+}
+
+// modes grouped by k1 and packed for one copy to the device: re, im, then the ints
+struct PackedGroups {
+    std::vector<char> blob;
+    size_t n = 0, groups = 0;
+
+    explicit PackedGroups(std::vector<HostMode> ms)
+    {
+        const auto less = [](const HostMode &a, const HostMode &b) {
+            return a.k1 != b.k1 ? a.k1 < b.k1 : a.k2 < b.k2;
+        };
+        if (!std::is_sorted(ms.begin(), ms.end(), less)) std::sort(ms.begin(), ms.end(), less);
+        n = ms.size();
+        for (size_t t = 0; t < n; ++t) groups += t == 0 || ms[t].k1 != ms[t - 1].k1;
+        blob.resize(n * 16 + (n + 2 * groups + 1) * 4);
+        double *re = reinterpret_cast<double *>(blob.data()), *im = re + n;
+        int *k2 = reinterpret_cast<int *>(im + n), *gk1 = k2 + n, *gofs = gk1 + groups;
+        size_t g = 0;
+        for (size_t t = 0; t < n; ++t) {
+            if (t == 0 || ms[t].k1 != ms[t - 1].k1) { gk1[g] = ms[t].k1; gofs[g++] = (int)t; }
+            k2[t] = ms[t].k2; re[t] = ms[t].re; im[t] = ms[t].im;
+        }
+        gofs[g] = (int)n;
+    }
+    // the groups as they lie in a device copy of the blob
+    ModeGroups at(void *dev) const
+    {
+        ModeGroups g;
+        g.n_groups = (int)groups;
+        double *re = static_cast<double *>(dev);
+        g.re = re;
+        g.im = re + n;
+        const int *k2 = reinterpret_cast<const int *>(re + 2 * n);
+        g.k2 = k2;
+        g.gk1 = k2 + n;
+        g.gofs = k2 + n + groups;
+        return g;
+    }
+};
+
+// group modes by k1 and upload: returns device ModeGroups pointing into one allocation of h
+int upload_groups(mlsd_levels *h, const std::vector<HostMode> &modes, ModeGroups &g)
+{
+    const PackedGroups pk(modes);
+    g = ModeGroups{};
+    if (modes.empty()) return MLSD_OK;
+    void *p = nullptr;
+    int rc = dev_alloc(h, &p, pk.blob.size());
+    if (rc) return rc;
+    CK(cudaMemcpy(p, pk.blob.data(), pk.blob.size(), cudaMemcpyHostToDevice));
+    g = pk.at(p);
     return MLSD_OK;
 }
 
@@ -241,13 +285,13 @@ int rule_sizes(mlsd_levels *h, DevLevel &d, const std::vector<HostMode> &diag, c
     if (!diag.empty()) {
         mlsd_levels tmp;                     // owns the set-up buffers of this step
         ModeGroups g1, g2;
-        int rc = upload_groups(&tmp, c1, g1);
-        if (!rc) rc = upload_groups(&tmp, c2, g2);
+        int rc = upload_groups(&tmp, fold_modes(c1), g1);
+        if (!rc) rc = upload_groups(&tmp, fold_modes(c2), g2);
         void *v1 = nullptr, *v2 = nullptr, *G = nullptr, *vmx = nullptr;
         cudaError_t e = cudaSuccess;
         if (!rc) e = cudaMalloc(&v1, (size_t)Nr * Nr * 8);
         if (!rc && e == cudaSuccess) e = cudaMalloc(&v2, (size_t)Nr * Nr * 8);
-        if (!rc && e == cudaSuccess) e = cudaMalloc(&G, (size_t)g1.n_groups * Nr * sizeof(double2));
+        if (!rc && e == cudaSuccess) e = cudaMalloc(&G, (size_t)(g1.n_groups + 1) * Nr * sizeof(double2));
         if (!rc && e == cudaSuccess) e = cudaMalloc(&vmx, (size_t)h->P * 8);
         if (!rc && e == cudaSuccess) e = launch_band_synth(g1, Nr, static_cast<double2 *>(G), v1, 1, s);
         if (!rc && e == cudaSuccess) e = launch_band_synth(g2, Nr, static_cast<double2 *>(G), v2, 1, s);
@@ -362,11 +406,11 @@ int build(const mlsd_problem *p, cudaStream_t s, mlsd_levels *h)
 
         // band grid of every class (set-up)
         ModeGroups g;
-        if ((rc = upload_groups(h, diag[l], g))) return rc;
+        if ((rc = upload_groups(h, fold_modes(diag[l]), g))) return rc;
         for (auto &c : d.cls) {
             if ((rc = dev_alloc(h, &c.band, (size_t)c.Nl * c.Nl * rs))) return rc;
             void *G = nullptr;
-            if (g.n_groups > 0) CK(cudaMalloc(&G, (size_t)g.n_groups * c.Nl * sizeof(double2)));
+            if (g.n_groups > 0) CK(cudaMalloc(&G, (size_t)(g.n_groups + 1) * c.Nl * sizeof(double2)));
             cudaError_t e = launch_band_synth(g, c.Nl, static_cast<double2 *>(G), c.band,
                                               p->precision == MLSD_FP64, s);
             if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1223,20 +1267,20 @@ int mlsd_grid_psi(int n_modes, const int32_t *k1, const int32_t *k2, const doubl
     if (n_modes < 0 || nf < 1 || !psi_dev || (n_modes > 0 && (!k1 || !k2 || !re || !im)))
         return MLSD_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    mlsd_levels tmp;   // owns the staging buffers for this call only
-    std::vector<HostMode> ms;
-    for (int t = 0; t < n_modes; ++t) ms.push_back({k1[t], k2[t], re[t], im[t]});
-    ModeGroups g;
-    int rc = upload_groups(&tmp, ms, g);
-    void *G = nullptr;
-    cudaError_t e = cudaSuccess;
-    if (!rc && g.n_groups > 0) e = cudaMalloc(&G, (size_t)g.n_groups * nf * sizeof(double2));
-    if (!rc && e == cudaSuccess) e = launch_band_synth(g, nf, static_cast<double2 *>(G), psi_dev, 0, s);
-    if (!rc && e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (G) cudaFree(G);
-    for (void *p : tmp.allocs) cudaFree(p);
-    if (rc) return rc;
-    CK(e);
+    std::vector<HostMode> ms((size_t)n_modes);
+    for (int t = 0; t < n_modes; ++t) ms[(size_t)t] = {k1[t], k2[t], re[t], im[t]};
+    // one workspace: the packed modes, then the synthesis' scratch
+    const PackedGroups pk(fold_modes(ms));
+    const size_t mb = (pk.blob.size() + 255) / 256 * 256;
+    const size_t gb = (pk.groups + 1) * (size_t)nf * sizeof(double2);
+    char *ws = nullptr;
+    CK(cudaMallocAsync((void **)&ws, mb + gb, s));
+    cudaError_t e = cudaMemcpyAsync(ws, pk.blob.data(), pk.blob.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+        e = launch_band_synth(pk.at(ws), nf, reinterpret_cast<double2 *>(ws + mb), psi_dev, 0, s);
+    cudaFreeAsync(ws, s);
+    const cudaError_t e2 = cudaStreamSynchronize(s);
+    CK(e == cudaSuccess ? e2 : e);
     return MLSD_OK;
 }
 
