@@ -5,8 +5,9 @@
 // mixed term by the 4-point average of cross differences (9-point stencil),
 // Heun's RK2.  Every face flux is evaluated by both adjacent cells with the
 // same operations, so sum(U) telescopes exactly apart from summation rounding.
-//   N <= 64: one persistent CTA keeps U, U* and K in shared memory for all steps.
-//   N  > 64: one launch per RK stage over the grid.
+// Small grids: one CTA keeps U and U* in shared memory and its face coefficients in
+// registers for all steps.  Larger ones: tiles, each CTA taking a tile with a halo
+// through several steps per launch (the halo's outer rings are recomputed).
 // The mass H^2 sum(U) of every step is summed in FP64.
 //
 // DNS: u_t = v1 D0x u + v2 D0y u + kappa (Dxx + Dyy) u, v = (-D0y psi, D0x psi),
@@ -26,40 +27,14 @@
 namespace mlsd {
 namespace {
 
-// DIR = false: periodic in both directions.  DIR = true: the Sec. 4 set-up,
-// Dirichlet in x1 -- column 0 is the boundary x1 = 0 (held by the caller) and
-// the virtual column N the boundary x1 = 2 pi with value ur; the K field stays
-// periodic (its column N is column 0).  Column 0 itself has no update (0).
-template <typename real, bool DIR = false>
-__device__ __forceinline__ real macro_rhs(int N, real invH, real inv4H, const real *U,
-                                          const real *K11, const real *K12, const real *K22,
-                                          int i, int j, real ur = (real)0)
+// Chains of launches that each read what the one before wrote: a kernel launched with
+// launch_chained starts while its predecessor still runs, loads what the predecessor does not
+// write (coefficients), and calls chain_wait before it reads or writes the fields.
+// The successor is let in only after that wait: one launch ahead, no further.
+__device__ __forceinline__ void chain_wait()
 {
-    if (DIR && i == 0) return (real)0;
-    const int ipk = (i + 1 == N) ? 0 : i + 1, im = (i == 0) ? N - 1 : i - 1;
-    const int jp = (j + 1 == N) ? 0 : j + 1, jm = (j == 0) ? N - 1 : j - 1;
-    const int c = j * N + i;
-    const bool edge = DIR && i + 1 == N;        // east neighbours are the boundary value
-    const real uE = edge ? ur : U[j * N + ipk], uEn = edge ? ur : U[jp * N + ipk];
-    const real uEs = edge ? ur : U[jm * N + ipk];
-    const real h = (real)0.5;
-    // east face (i+1/2, j)
-    real k11 = h * (K11[c] + K11[j * N + ipk]), k12 = h * (K12[c] + K12[j * N + ipk]);
-    const real fe = k11 * (uE - U[c]) * invH
-                  + k12 * (U[jp * N + i] + uEn - U[jm * N + i] - uEs) * inv4H;
-    // west face (i-1/2, j)
-    k11 = h * (K11[j * N + im] + K11[c]); k12 = h * (K12[j * N + im] + K12[c]);
-    const real fw = k11 * (U[c] - U[j * N + im]) * invH
-                  + k12 * (U[jp * N + im] + U[jp * N + i] - U[jm * N + im] - U[jm * N + i]) * inv4H;
-    // north face (i, j+1/2)
-    real k22 = h * (K22[c] + K22[jp * N + i]); k12 = h * (K12[c] + K12[jp * N + i]);
-    const real fn = k22 * (U[jp * N + i] - U[c]) * invH
-                  + k12 * (uE + uEn - U[j * N + im] - U[jp * N + im]) * inv4H;
-    // south face (i, j-1/2)
-    k22 = h * (K22[jm * N + i] + K22[c]); k12 = h * (K12[jm * N + i] + K12[c]);
-    const real fs = k22 * (U[c] - U[jm * N + i]) * invH
-                  + k12 * (uEs + uE - U[jm * N + im] - U[j * N + im]) * inv4H;
-    return (fe - fw + fn - fs) * invH;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // deterministic FP64 block sum (all threads return the total)
@@ -74,84 +49,227 @@ __device__ double block_sum(double v, double *red)
     return t;
 }
 
-// one CTA, everything in shared memory (DIR: column 0 set to ul, east boundary ur)
-template <typename real, bool DIR = false>
-__global__ void __launch_bounds__(1024) k_macro_resident(int N, real *Ug, const double *Kg,
-                                                         real dt, int nsteps, double *mass,
-                                                         real ul = (real)0, real ur = (real)0)
+// Face coefficients of the flux form, scaled by dt / H: with the face tensors
+// K_f = (K_node + K_neighbour) / 2, the east face (i+1/2, j) of cell (i, j) carries
+//   fe = aE (uE - u) + cE (Dc + DE),   aE = dt K11_f / H^2, cE = dt K12_f / (4 H^2),
+// D = u(j+1) - u(j-1) of a column, the north face (i, j+1/2)
+//   fn = aN (uN - u) + cN (Gc + GN),   aN = dt K22_f / H^2, cN = dt K12_f / (4 H^2),
+// G = u(i+1) - u(i-1) of a row, and dt div(K grad U) = (fe - fw) + (fn - fs), the west and
+// south fluxes being the neighbours' east and north ones formed from the same operands.
+// Coefficient q (0: aE, 1: cE, 2: aN, 3: cN) of cell (i, j) from the node tensors; f = dt / (2 H^2)
+template <typename real>
+__device__ __forceinline__ real macro_face(int q, const double *Kg, int N, int i, int j, real f)
+{
+    const int c = j * N + i;
+    const int o = q < 2 ? j * N + (i + 1 == N ? 0 : i + 1) : (j + 1 == N ? 0 : j + 1) * N + i;
+    const int k = q == 0 ? 0 : (q == 2 ? 2 : 1);
+    return ((q & 1) ? (real)0.25 * f : f) * ((real)Kg[3 * c + k] + (real)Kg[3 * o + k]);
+}
+
+// coefficients into co [4][N][N]; U into V when V is given; with dir, column 0 of U (and V)
+// takes the boundary value ul
+template <typename real>
+__global__ void k_macro_prep(int N, const double *Kg, real f, real *co, real *U, real *V, int dir,
+                             real ul)
+{
+    const int c = blockIdx.x * blockDim.x + threadIdx.x, NN = N * N;
+    if (c >= NN) return;
+    const int i = c % N, j = c / N;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) co[q * NN + c] = macro_face(q, Kg, N, i, j, f);
+    if (dir && i == 0) U[c] = ul;
+    if (V) V[c] = (dir && i == 0) ? ul : U[c];
+}
+
+// The R cells (x, y0 .. y0+R-1) of a thread: their coefficients, and one Heun stage.
+template <typename real, int R>
+struct MacroStrip {
+    real aE[R], cE[R], aW[R], cW[R], aN[R + 1], cN[R + 1];   // aN[r]: south face of row r
+
+    // coefficients co(q, i, j) of the cells at columns gx (west neighbour gw) and rows gy(r),
+    // r = -1 .. R-1
+    template <typename Co, typename Row>
+    __device__ __forceinline__ void load(Co co, int gx, int gw, Row gy)
+    {
+#pragma unroll
+        for (int r = 0; r <= R; ++r) {
+            const int j = gy(r - 1);
+            aN[r] = co(2, gx, j);
+            cN[r] = co(3, gx, j);
+            if (r > 0) {
+                aE[r - 1] = co(0, gx, j); cE[r - 1] = co(1, gx, j);
+                aW[r - 1] = co(0, gw, j); cW[r - 1] = co(1, gw, j);
+            }
+        }
+    }
+
+    // out[r] = dt div(K grad X) of the strip's cells; X(row r = -1 .. R, column -1 | 0 | 1)
+    template <typename Get>
+    __device__ __forceinline__ void rhs(Get X, real (&out)[R]) const
+    {
+        real wm = X(-1, -1), cm = X(-1, 0), em = X(-1, 1);
+        real w = X(0, -1), c = X(0, 0), e = X(0, 1);
+        real g = e - w;
+        // south flux of row 0
+        real fs = fma(aN[0], c - cm, cN[0] * (g + (em - wm)));
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const real wp = X(r + 1, -1), cp = X(r + 1, 0), ep = X(r + 1, 1);
+            const real Dw = wp - wm, Dc = cp - cm, De = ep - em, gp = ep - wp;
+            const real fe = fma(aE[r], e - c, cE[r] * (Dc + De));
+            const real fw = fma(aW[r], c - w, cW[r] * (Dc + Dw));
+            const real fn = fma(aN[r + 1], cp - c, cN[r + 1] * (g + gp));
+            out[r] = (fe - fw) + (fn - fs);
+            fs = fn;
+            wm = w; cm = c; em = e;
+            w = wp; c = cp; e = ep;
+            g = gp;
+        }
+    }
+};
+
+// One CTA, the whole grid in shared memory for all steps, a thread a cell with its eight face
+// coefficients in registers.  DIR: the Sec. 4 set-up, Dirichlet in x1 -- column 0 is the
+// boundary x1 = 0 (held) and the virtual column N the boundary x1 = 2 pi with value ur; the K
+// field stays periodic.
+template <typename real, int NT, bool DIR>
+__global__ void __launch_bounds__(NT) k_macro_resident(int N, real *Ug, const double *Kg, real f,
+                                                       int nsteps, double *mass, real ul, real ur)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    real *U = reinterpret_cast<real *>(smem_raw);
-    real *Us = U + N * N, *K11 = Us + N * N, *K12 = K11 + N * N, *K22 = K12 + N * N;
+    real *U = reinterpret_cast<real *>(smem_raw), *Us = U + N * N;
     __shared__ double red[32];
-    const int NN = N * N;
-    const double H = 2.0 * kPi / N;
-    const real invH = (real)(1.0 / H), inv4H = (real)(1.0 / (4.0 * H));
-    const double H2 = H * H;
+    const int c = threadIdx.x, x = c % N, y = c / N;
+    const bool own = y < N;
+    const double H = 2.0 * kPi / N, H2 = H * H;
+    const int xe = x + 1 == N ? 0 : x + 1, xw = x == 0 ? N - 1 : x - 1;
+    const int yn = y + 1 >= N ? 0 : y + 1, ys = y == 0 ? N - 1 : y - 1;
+    const bool held = DIR && x == 0, east = DIR && x + 1 == N;
+    MacroStrip<real, 1> st;
+    real u = 0, d[1], s;
     double m = 0.0;
-    for (int c = threadIdx.x; c < NN; c += blockDim.x) {
-        U[c] = (DIR && c % N == 0) ? ul : Ug[c];
-        K11[c] = (real)Kg[3 * c]; K12[c] = (real)Kg[3 * c + 1]; K22[c] = (real)Kg[3 * c + 2];
-        m += (double)U[c];
+    if (own) {
+        st.load([&](int q, int i, int j) { return macro_face(q, Kg, N, i, j, f); }, x, xw,
+                [&](int r) { return r < 0 ? ys : y; });
+        u = held ? ul : Ug[c];
+        U[c] = u;
+        m = (double)u;
     }
     m = block_sum(m, red);
     if (threadIdx.x == 0 && mass) mass[0] = m * H2;
-    for (int s = 1; s <= nsteps; ++s) {
-        for (int c = threadIdx.x; c < NN; c += blockDim.x)
-            Us[c] = U[c] + dt * macro_rhs<real, DIR>(N, invH, inv4H, U, K11, K12, K22, c % N, c / N, ur);
+    const int row[3] = {ys * N, y * N, yn * N};
+    auto stage = [&](const real *X) {
+        st.rhs([&](int r, int k) {
+            return k == 0 ? X[row[r + 1] + x] : k < 0 ? X[row[r + 1] + xw] : (east ? ur : X[row[r + 1] + xe]);
+        }, d);
+    };
+    for (int k = 1; k <= nsteps; ++k) {
+        if (own) {
+            stage(U);
+            s = held ? u : u + d[0];
+            Us[c] = s;
+        }
         __syncthreads();
-        real nu[4];
-        int k = 0;
-        for (int c = threadIdx.x; c < NN; c += blockDim.x, ++k)
-            nu[k] = (real)0.5 * (U[c] + Us[c] + dt * macro_rhs<real, DIR>(N, invH, inv4H, Us, K11, K12, K22, c % N, c / N, ur));
-        __syncthreads();
-        k = 0;
         m = 0.0;
-        for (int c = threadIdx.x; c < NN; c += blockDim.x, ++k) { U[c] = nu[k]; m += (double)nu[k]; }
+        if (own) {
+            stage(Us);
+            u = held ? u : (real)0.5 * (u + s + d[0]);
+            U[c] = u;
+            m = (double)u;
+        }
         if (mass) {
             m = block_sum(m, red);
-            if (threadIdx.x == 0) mass[s] = m * H2;
-        } else {
-            __syncthreads();
+            if (threadIdx.x == 0) mass[k] = m * H2;
         }
+        __syncthreads();
     }
-    for (int c = threadIdx.x; c < NN; c += blockDim.x) Ug[c] = U[c];
+    if (own) Ug[c] = u;
 }
 
-template <typename real>
-__global__ void k_split_K(int NN, const double *Kg, real *K11, real *K12, real *K22)
+// `steps` <= S Heun steps of one TX x TY tile per CTA.  The tile comes with a halo of 2 S
+// cells; each stage is valid on one ring less, so strips of R rows outside a stage's valid
+// rows are skipped, the rest of the rim is computed with clamped neighbours and never
+// stored.  What bounds it: latency (a launch, two barriers a step), in FP64 issue beside it.
+// A step at 128^2: FP32 1.14 us, against 10.0 with a launch per Heun stage that formed every
+// face from K again, 1.54 without overlapping the launches; FP64 5.2 us against 16.6.
+// With part, the tile's share of sum(U) after step k goes to
+// part[k * tiles + tile].
+template <typename real, int TX, int TY, int S, bool DIR>
+struct MacroTile {
+    static constexpr int HALO = 2 * S, EX = TX + 2 * HALO, EY = TY + 2 * HALO;
+    static constexpr int R = sizeof(real) == 8 ? 1 : 4;
+    static constexpr int NT = EX * EY / R;
+    static_assert(EY % R == 0 && NT <= 1024, "strips of R rows");
+};
+template <typename real, int TX, int TY, int S, bool DIR>
+__global__ void __launch_bounds__((MacroTile<real, TX, TY, S, DIR>::NT + 31) / 32 * 32)
+k_macro_tile(int N, const real *Uin, real *Uout, const real *__restrict__ co,
+             int steps, double *part, real ur)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= NN) return;
-    K11[c] = (real)Kg[3 * c]; K12[c] = (real)Kg[3 * c + 1]; K22[c] = (real)Kg[3 * c + 2];
-}
-
-// stage 1: Us = U + dt R(U); stage 2: U = (U + Us + dt R(Us)) / 2, with the block's
-// share of sum(U) written to part[block]
-template <typename real, bool SECOND, bool DIR = false>
-__global__ void k_macro_stage(int N, real *U, real *Us, const real *K11, const real *K12,
-                              const real *K22, real dt, double *part, real ur = (real)0)
-{
+    using M = MacroTile<real, TX, TY, S, DIR>;
+    constexpr int EX = M::EX, EY = M::EY, R = M::R, HALO = M::HALO;
+    __shared__ real U[EY * EX], Us[EY * EX];
     __shared__ double red[32];
-    const int NN = N * N;
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    const double H = 2.0 * kPi / N;
-    const real invH = (real)(1.0 / H), inv4H = (real)(1.0 / (4.0 * H));
-    double m = 0.0;
-    if (c < NN) {
-        if (!SECOND) {
-            Us[c] = U[c] + dt * macro_rhs<real, DIR>(N, invH, inv4H, U, K11, K12, K22, c % N, c / N, ur);
-        } else {
-            const real v = (real)0.5 * (U[c] + Us[c] + dt * macro_rhs<real, DIR>(N, invH, inv4H, Us, K11, K12, K22, c % N, c / N, ur));
-            m = (double)v;
-            // U is read by neighbours only in stage 1, so the in-place write is safe here
-            U[c] = v;
+    const int t = threadIdx.x, x = t % EX, y0 = t / EX * R;
+    const bool own = t < M::NT;                     // the last warp may be partial
+    const int gx0 = blockIdx.x * TX - HALO + x;     // grid column before the periodic wrap
+    const int gx = ((gx0 % N) + N) % N, gw = gx == 0 ? N - 1 : gx - 1;
+    auto gy = [&](int r) { const int y = (int)blockIdx.y * TY - HALO + y0 + r; return ((y % N) + N) % N; };
+    const bool held = DIR && (gx0 == 0 || gx0 == N);
+    MacroStrip<real, R> st;
+    real u[R], d[R], s[R];
+    if (own) st.load([&](int q, int i, int j) { return co[((long long)q * N + j) * N + i]; }, gx, gw, gy);
+    chain_wait();
+    if (own) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            u[r] = (DIR && gx0 == N) ? ur : Uin[(long long)gy(r) * N + gx];
+            U[(y0 + r) * EX + x] = u[r];
         }
     }
-    if (SECOND && part) {
-        m = block_sum(m, red);
-        if (threadIdx.x == 0) part[blockIdx.x] = m;
+    // cells of the tile that are inside the grid
+    const bool colin = own && x >= HALO && x < HALO + TX && gx0 < N;
+    auto inside = [&](int r) {
+        return colin && y0 + r >= HALO && y0 + r < HALO + TY && (int)blockIdx.y * TY - HALO + y0 + r < N;
+    };
+    __syncthreads();
+    const int xw = x > 0 ? -1 : 0, xe = x < EX - 1 ? 1 : 0;
+    const int ym = y0 > 0 ? y0 - 1 : 0, yp = y0 + R < EY ? y0 + R : EY - 1;
+    auto stage = [&](const real *X) {
+        st.rhs([&](int r, int k) {
+            return X[(r < 0 ? ym : r == R ? yp : y0 + r) * EX + x + (k < 0 ? xw : k > 0 ? xe : 0)];
+        }, d);
+    };
+    for (int k = 0; k < steps; ++k) {
+        if (own && y0 + R > 2 * k + 1 && y0 < EY - 1 - 2 * k) {
+            stage(U);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                s[r] = held ? u[r] : u[r] + d[r];
+                Us[(y0 + r) * EX + x] = s[r];
+            }
+        }
+        __syncthreads();
+        double m = 0.0;
+        if (own && y0 + R > 2 * k + 2 && y0 < EY - 2 - 2 * k) {
+            stage(Us);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                u[r] = held ? u[r] : (real)0.5 * (u[r] + s[r] + d[r]);
+                U[(y0 + r) * EX + x] = u[r];
+                if (part && inside(r)) m += (double)u[r];
+            }
+        }
+        if (part) {
+            m = block_sum(m, red);
+            if (t == 0)
+                part[(long long)k * gridDim.x * gridDim.y + blockIdx.y * gridDim.x + blockIdx.x] = m;
+        }
+        __syncthreads();
     }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        if (inside(r)) Uout[(long long)gy(r) * N + gx] = u[r];
 }
 
 // Dirichlet set-up: column 0 (the boundary x1 = 0) takes the boundary value
@@ -662,49 +780,92 @@ __global__ void k_sum(int n, const double *x, double scale, double *out)
 
 }  // namespace
 
+// Which kernel takes an N x N grid: one CTA for the whole run up to 32^2 in FP32 and 16^2 in
+// FP64 (where one SM's 2 FP64 operations a clock decide), tiles above.  A step, resident
+// against tiles: FP32 0.83 us at 32^2 (tiles 1.1 at every side up to 128); FP64 4.05 us at 16^2
+// and 6.5 at 20^2 (tiles 4.8 - 5.2 at sides 24 to 128).
+static bool macro_resident(int N, int precision) { return N <= (precision == MLSD_FP64 ? 16 : 32); }
+// tiles: 16 x 16 cells and 4 steps a launch in FP32; 16 x 8 cells and 1 step in FP64, where
+// the recomputed halo costs more than a launch
+constexpr int kTileX = 16, kTileY32 = 16, kSteps32 = 4, kTileY64 = 8, kSteps64 = 1;
+static long long macro_tiles(int N, int precision)
+{
+    const int ty = precision == MLSD_FP64 ? kTileY64 : kTileY32;
+    return (long long)((N + kTileX - 1) / kTileX) * ((N + ty - 1) / ty);
+}
+static long long macro_mass_blocks(int N, int precision)
+{
+    return std::max(((long long)N * N + 255) / 256, macro_tiles(N, precision));
+}
+
+// launch a kernel of a chain; overlap: let it start before its predecessor in the stream ends
+template <typename... P, typename... A>
+static cudaError_t launch_chained(void (*fn)(P...), dim3 grid, int threads, bool overlap, cudaStream_t s,
+                                  A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, fn, P(args)...);
+}
+
 size_t macro_scratch_bytes(int N, int precision, int nsteps)
 {
     const size_t rs = precision == MLSD_FP64 ? 8 : 4;
     const size_t NN = (size_t)N * N;
-    if (N <= 64) return 0;
-    const size_t nblocks = (NN + 255) / 256;
-    return 4 * NN * rs + 256 + (size_t)(nsteps + 1) * nblocks * sizeof(double);
+    if (macro_resident(N, precision)) return 0;
+    return 5 * NN * rs + 256 + (size_t)(nsteps + 1) * macro_mass_blocks(N, precision) * sizeof(double);
 }
 
 template <typename real, bool DIR>
 static cudaError_t macro_run_t(int N, real *U, const double *K, double dt, int nsteps,
                                double *mass, void *scratch, cudaStream_t s, double ul, double ur)
 {
-    const int NN = N * N;
+    constexpr bool F64 = sizeof(real) == 8;
+    constexpr int prec = F64 ? MLSD_FP64 : MLSD_FP32;
+    const int NN = N * N, th = 256, nb = (NN + th - 1) / th;
     const double H = 2.0 * kPi / N;
-    if (N <= 64) {
-        const size_t smem = 5 * (size_t)NN * sizeof(real);
-        cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&k_macro_resident<real, DIR>),
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        const int threads = NN >= 1024 ? 1024 : ((NN + 31) / 32) * 32;
+    const real f = (real)(0.5 * dt / (H * H)), l = (real)ul, r = (real)ur;
+    if (macro_resident(N, prec)) {
+        const int threads = (NN + 31) / 32 * 32;
         count_launches(1);
-        k_macro_resident<real, DIR><<<1, threads, smem, s>>>(N, U, K, (real)dt, nsteps, mass,
-                                                             (real)ul, (real)ur);
+        k_macro_resident<real, F64 ? 256 : 1024, DIR><<<1, threads, 2 * (size_t)NN * sizeof(real), s>>>(
+            N, U, K, f, nsteps, mass, l, r);
         return cudaGetLastError();
     }
-    real *Us = static_cast<real *>(scratch);
-    real *K11 = Us + NN, *K12 = K11 + NN, *K22 = K12 + NN;
-    const int th = 256, nb = (NN + th - 1) / th;
+    real *co = static_cast<real *>(scratch), *V = co + 4 * (size_t)NN;
+    constexpr int S = F64 ? kSteps64 : kSteps32, TY = F64 ? kTileY64 : kTileY32;
+    const int launches = (nsteps + S - 1) / S;
+    // the tile launches ping-pong between U and V and end in U
+    const bool start_in_V = launches & 1;
+    count_launches(1);
+    k_macro_prep<real><<<nb, th, 0, s>>>(N, K, f, co, U, start_in_V ? V : nullptr, DIR ? 1 : 0, l);
     double *part = reinterpret_cast<double *>(
-        (reinterpret_cast<uintptr_t>(K22 + NN) + 255) & ~(uintptr_t)255);
-    count_launches(1 + 2 * (long long)nsteps + (mass ? 2 : 0) + (DIR ? 1 : 0));
-    k_split_K<real><<<nb, th, 0, s>>>(NN, K, K11, K12, K22);
-    if (DIR) k_set_col0<real><<<(N + 255) / 256, 256, 0, s>>>(N, U, (real)ul);
+        (reinterpret_cast<uintptr_t>(V + NN) + 255) & ~(uintptr_t)255);
+    using T = MacroTile<real, kTileX, TY, S, DIR>;
+    const dim3 grid((N + kTileX - 1) / kTileX, (N + TY - 1) / TY);
+    const long long tiles = (long long)grid.x * grid.y, stride = macro_mass_blocks(N, prec);
+    count_launches(launches + (mass ? 3 : 0));
     if (mass) k_mass_part<real><<<nb, th, 0, s>>>(NN, U, part);
-    for (int st = 1; st <= nsteps; ++st) {
-        k_macro_stage<real, false, DIR><<<nb, th, 0, s>>>(N, U, Us, K11, K12, K22, (real)dt, nullptr,
-                                                          (real)ur);
-        k_macro_stage<real, true, DIR><<<nb, th, 0, s>>>(N, U, Us, K11, K12, K22, (real)dt,
-                                                         mass ? part + (size_t)st * nb : nullptr,
-                                                         (real)ur);
+    real *a = start_in_V ? V : U, *b = start_in_V ? U : V;
+    for (int k = 0; k < nsteps; k += S) {
+        const cudaError_t e = launch_chained(
+            k_macro_tile<real, kTileX, TY, S, DIR>, grid, (T::NT + 31) / 32 * 32, k > 0, s, N, a, b, co,
+            std::min(S, nsteps - k), mass ? part + stride + (size_t)k * tiles : nullptr, r);
+        if (e != cudaSuccess) return e;
+        std::swap(a, b);
     }
-    if (mass) k_mass_final<<<(nsteps + 1 + 127) / 128, 128, 0, s>>>(nsteps + 1, nb, part, H * H, mass);
+    if (mass) {
+        k_mass_final<<<1, 128, 0, s>>>(1, nb, part, H * H, mass);
+        if (nsteps > 0)
+            k_mass_final<<<(nsteps + 127) / 128, 128, 0, s>>>(nsteps, (int)tiles, part + stride, H * H, mass + 1);
+    }
     return cudaGetLastError();
 }
 
