@@ -699,37 +699,180 @@ __global__ void k_wait_check_tile(int *status)
     }
 }
 
-// DNS with the Sec. 4 boundaries (Dirichlet in x1, periodic in x2): one launch
-// per Heun stage, one thread per node.  Column 0 is the boundary x1 = 0 (held
-// at ul), the virtual column nf the boundary x1 = 2 pi (value ur); psi and the
-// velocity stay periodic.  Stage 1: s = u + dt f(u) into `out`; stage 2:
-// out = (u + s + dt f(s)) / 2 with `s` the stage-1 field.  The same folded
-// constants as k_dns_step: cA = dt / (4 h^2) on psi differences times u
-// differences, cD = dt kappa / h^2 on the Laplacian (kept as a difference).
-template <bool SECOND, typename real>
-__global__ void k_dns_dir_stage(int nf, const real *__restrict__ u, const real *__restrict__ sfield,
-                                const float *__restrict__ psi, real *__restrict__ out, real cA,
-                                real cD, real ul, real ur)
+// Several Heun steps of one tile per CTA (FP32): grids that the chip's L2 holds, where a
+// launch per step is mostly latency.  The tile comes with a halo of 2 S cells and the whole
+// run of `steps` <= S steps stays on chip; each stage is valid on one ring less, so strips
+// outside a stage's valid rows are skipped and the rest of the rim is computed with clamped
+// neighbours and never stored.  A thread owns R rows of one column: its cells and the psi
+// differences that multiply them live in registers, the field goes through shared memory
+// once per stage.  The arithmetic per cell is dns_tile's, operand for operand:
+//   x + dt f(x) = x + cD (xE + xW + xN + xS - 4 x)
+//                   + cA [(psiS - psiN)(xE - xW) + (psiE - psiW)(xN - xS)].
+// DIR: Dirichlet in x1 (column 0 held at ul, the virtual column nf at ur), periodic in x2;
+// psi and the velocity stay periodic.  What bounds it: at 512^2 latency and FP32 issue (242
+// CTAs of 640 threads, 1.7 times the tile's cells); 1.8 us a step against 8.2 with a launch
+// per Heun stage (Dirichlet) and 6.2 for the per-tile kernel (periodic).
+template <int EX, int EY, int S, int R>
+struct DnsSteps {
+    static constexpr int HALO = 2 * S, TX = EX - 2 * HALO, TY = EY - 2 * HALO, NT = EX * (EY / R);
+    static_assert(EX % 32 == 0 && EY % R == 0 && NT <= 1024 && TX > 0 && TY > 0, "whole strips");
+};
+template <int EX, int EY, int S, int R, bool DIR>
+__global__ void __launch_bounds__(DnsSteps<EX, EY, S, R>::NT)
+k_dns_steps(int nf, const float *uin, const float *__restrict__ psi, float *uout,
+            float cA, float cD, int steps, float ul, float ur)
+{
+    using D = DnsSteps<EX, EY, S, R>;
+    __shared__ float A[EY * EX], Bf[EY * EX];
+    const int x = threadIdx.x % EX, y0 = threadIdx.x / EX * R;
+    const int gx0 = (int)blockIdx.x * D::TX - D::HALO + x, gy0 = (int)blockIdx.y * D::TY - D::HALO + y0;
+    auto wrap = [&](int i) { return ((i % nf) + nf) % nf; };
+    const int gx = wrap(gx0);
+    const bool held = DIR && (gx0 == 0 || gx0 == nf);
+    float u[R], s[R], pa[R], pb[R];              // u, stage value, psiS - psiN, psiE - psiW
+    {
+        const int ge = gx + 1 == nf ? 0 : gx + 1, gw = gx == 0 ? nf - 1 : gx - 1;
+        float pc[R + 2];
+#pragma unroll
+        for (int r = -1; r <= R; ++r) pc[r + 1] = psi[(long long)wrap(gy0 + r) * nf + gx];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const long long row = (long long)wrap(gy0 + r) * nf;
+            pa[r] = pc[r] - pc[r + 2];
+            pb[r] = psi[row + ge] - psi[row + gw];
+        }
+        chain_wait();
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            u[r] = !held ? uin[(long long)wrap(gy0 + r) * nf + gx] : (gx0 == 0 ? ul : ur);
+            A[(y0 + r) * EX + x] = u[r];
+        }
+    }
+    __syncthreads();
+    const int xw = x > 0 ? x - 1 : 0, xe = x < EX - 1 ? x + 1 : EX - 1;
+    const int ym = y0 > 0 ? y0 - 1 : 0, yp = y0 + R < EY ? y0 + R : EY - 1;
+    // g = x + dt f(x) of this thread's cells c, the field in X
+    auto stage = [&](const float *X, const float (&c)[R], float (&g)[R]) {
+        const float below = X[ym * EX + x], above = X[yp * EX + x];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float W = X[(y0 + r) * EX + xw], E = X[(y0 + r) * EX + xe];
+            const float N = r + 1 < R ? c[(r + 1) % R] : above, B = r > 0 ? c[(r + R - 1) % R] : below;
+            float t = pa[r] * (E - W);
+            t = fmaf(pb[r], N - B, t);
+            const float lap = fmaf(-4.0f, c[r], (E + W) + (N + B));
+            g[r] = fmaf(cA, t, fmaf(cD, lap, c[r]));
+        }
+    };
+    for (int k = 0; k < steps; ++k) {
+        float g[R];
+        // rows 2k+1 .. EY-2-2k are valid after this stage
+        if (y0 + R > 2 * k + 1 && y0 < EY - 1 - 2 * k) {
+            stage(A, u, g);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                s[r] = held ? u[r] : g[r];
+                Bf[(y0 + r) * EX + x] = s[r];
+            }
+        }
+        __syncthreads();
+        if (y0 + R > 2 * k + 2 && y0 < EY - 2 - 2 * k) {
+            stage(Bf, s, g);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                u[r] = held ? u[r] : 0.5f * (u[r] + g[r]);
+                A[(y0 + r) * EX + x] = u[r];
+            }
+        }
+        __syncthreads();
+    }
+    if (x >= D::HALO && x < D::HALO + D::TX && gx0 < nf)
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (y0 + r >= D::HALO && y0 + r < D::HALO + D::TY && gy0 + r < nf)
+                uout[(long long)(gy0 + r) * nf + gx0] = u[r];
+}
+
+// FP64 Dirichlet runs.  What bounds them is FP64 issue (2 operations a clock and SM), so the
+// step is written with as few as possible: with A = dt f's linear part, Heun's step of this
+// linear problem is u + A u + A^2 u / 2 = u + A' (s), s = sqrt2 u + A' u, A' = A / sqrt2, and
+//   A' x = aE xE + aW xW + aN xN + aS xS - 4 d x,   d = dt kappa / (sqrt2 h^2),
+//   aE, aW = d +- c1, aN, aS = d +- c2,  c1, c2 = dt / (4 sqrt2 h^2) (psiS - psiN, psiE - psiW):
+// 5 operations a cell and stage, none of them a conversion (aE and aN come from arrays formed
+// once per run; 12 operations and 4 conversions a cell and stage before).  512^2: 9.8 us a step
+// against 24.7 with a launch per stage.  The boundary values enter the first stage scaled by sqrt2.
+__global__ void k_dns_dir_coef(int nf, const float *__restrict__ psi, double cA, double d,
+                               double *__restrict__ aE, double *__restrict__ aN)
 {
     const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (c >= (long long)nf * nf) return;
     const int a = (int)(c % nf), b = (int)(c / nf);
-    if (a == 0) { out[c] = ul; return; }
-    const real *x = SECOND ? sfield : u;
     const int bp = b + 1 == nf ? 0 : b + 1, bm = b == 0 ? nf - 1 : b - 1;
-    const int ap = a + 1 == nf ? 0 : a + 1;
+    const int ap = a + 1 == nf ? 0 : a + 1, am = a == 0 ? nf - 1 : a - 1;
     const long long row = (long long)b * nf;
-    const real xc = x[c];
-    const real xE = a + 1 == nf ? ur : x[row + ap], xW = x[c - 1];
-    const real xN = x[(long long)bp * nf + a], xS = x[(long long)bm * nf + a];
-    // dt (v1 D0x + v2 D0y) x = cA [(psiS - psiN)(xE - xW) + (psiE - psiW)(xN - xS)]
-    const real pN = psi[(long long)bp * nf + a], pS = psi[(long long)bm * nf + a];
-    const real pE = psi[row + ap], pW = psi[row + a - 1];
-    real t = (pS - pN) * (xE - xW);
-    t = fma(pE - pW, xN - xS, t);
-    const real lap = fma((real)-4, xc, (xE + xW) + (xN + xS));
-    const real g = fma(cA, t, fma(cD, lap, xc));
-    out[c] = SECOND ? (real)0.5 * (u[c] + g) : g;
+    aE[c] = fma(cA, (double)psi[(long long)bm * nf + a] - (double)psi[(long long)bp * nf + a], d);
+    aN[c] = fma(cA, (double)psi[row + ap] - (double)psi[row + am], d);
+}
+
+// One step of a 28 x TY tile per CTA, halo 2: a warp owns R rows of the 32 extended columns
+// (east and west neighbours by shuffles), rows outside a stage's valid ones are skipped.
+constexpr int kD64R = 2, kD64TX = 28;
+template <int TY>
+__global__ void __launch_bounds__(32 * (TY + 4) / kD64R)
+k_dns_dir_step64(int nf, const double *uin, double *uout, const double *__restrict__ aEg,
+                 const double *__restrict__ aNg, double d, double ul, double ur, double ul_s, double ur_s)
+{
+    constexpr int R = kD64R, EY = TY + 4;
+    __shared__ double A[EY * 32], Bf[EY * 32];
+    const int x = threadIdx.x & 31, y0 = (threadIdx.x >> 5) * R;
+    const int gx0 = (int)blockIdx.x * kD64TX - 2 + x, gy0 = (int)blockIdx.y * TY - 2 + y0;
+    auto wrap = [&](int i) { return ((i % nf) + nf) % nf; };
+    const int gx = wrap(gx0);
+    const bool held = gx0 == 0 || gx0 == nf;
+    const double two_d = 2.0 * d, m4d = -4.0 * d;
+    double u[R], aE[R], aN[R], aW[R], aS[R], s[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const long long c = (long long)wrap(gy0 + r) * nf + gx;
+        aE[r] = aEg[c];
+        aN[r] = aNg[c];
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) { aW[r] = two_d - aE[r]; aS[r] = two_d - aN[r]; }
+    chain_wait();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        u[r] = !held ? uin[(long long)wrap(gy0 + r) * nf + gx] : (gx0 == 0 ? ul : ur);
+        A[(y0 + r) * 32 + x] = u[r];
+    }
+    __syncthreads();
+    // acc + A' x without the centre term, c this thread's rows of the field in X
+    auto ring = [&](const double *X, const double (&c)[R], int r, double acc) {
+        const double E = __shfl_down_sync(0xffffffffu, c[r], 1), W = __shfl_up_sync(0xffffffffu, c[r], 1);
+        const double N = r + 1 < R ? c[(r + 1) % R] : X[(y0 + R < EY ? y0 + R : EY - 1) * 32 + x];
+        const double B = r > 0 ? c[(r + R - 1) % R] : X[(y0 > 0 ? y0 - 1 : 0) * 32 + x];
+        acc = fma(aE[r], E, acc);
+        acc = fma(aW[r], W, acc);
+        acc = fma(aN[r], N, acc);
+        return fma(aS[r], B, acc);
+    };
+    // stage 1 on rows 1 .. EY-2 (the strips at the rim compute theirs with a clamped row)
+    const double centre = 1.4142135623730951 + m4d;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const double g = ring(A, u, r, centre * u[r]);
+        s[r] = !held ? g : (gx0 == 0 ? ul_s : ur_s);
+        Bf[(y0 + r) * 32 + x] = s[r];
+    }
+    __syncthreads();
+    // stage 2 and the store: the strips of the tile's own rows
+    if (y0 < 2 || y0 >= EY - 2) return;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const double g = ring(Bf, s, r, fma(m4d, s[r], u[r]));
+        if (x >= 2 && x < 2 + kD64TX && gx0 < nf && gy0 + r < nf)
+            uout[(long long)(gy0 + r) * nf + gx0] = held ? u[r] : g;
+    }
 }
 
 // max over the grid of |v1| + |v2| (non-negative floats order like their bit patterns)
@@ -978,6 +1121,7 @@ static cudaError_t dns_launch_tma(int nf, const CUtensorMap &ma, const CUtensorM
 // two staging buffers, 64 rows with one; 32 rows with the f32x2 pair arithmetic).
 // Picked once per process by timing each on the caller's grid;
 // MLSD_DNS_TY = 64 | 32 | t32 | t32x2 | t64 | t32p pins one.
+static bool g_dns_multi = false;                 // the last run took several steps a launch
 enum DnsKind { kCp64, kCp32, kTma32, kTma32x2, kTma64, kTma32p, kDnsKinds };
 static int g_dns_kind = -1;
 
@@ -997,12 +1141,48 @@ static cudaError_t dns_launch_kind(int kind, int nf, const CUtensorMap *maps, in
     return cudaErrorInvalidValue;
 }
 
+// nsteps steps by k_dns_steps launches that ping-pong between u and u_tmp, ending in u
+template <bool DIR>
+static cudaError_t dns_multi(int nf, float *u, float *u_tmp, const float *psi, float cA, float cD,
+                             int nsteps, float ul, float ur, cudaStream_t s)
+{
+    constexpr int EX = 64, EY = 40, S = 4, R = 4;
+    using D = DnsSteps<EX, EY, S, R>;
+    // an even number of launches, the steps spread evenly over them (one step: a copy back)
+    int launches = (nsteps + S - 1) / S;
+    if ((launches & 1) && nsteps > 1) ++launches;
+    const dim3 grid((unsigned)((nf + D::TX - 1) / D::TX), (unsigned)((nf + D::TY - 1) / D::TY));
+    count_launches(launches);
+    float *a = u, *b = u_tmp;
+    for (int k = 0, done = 0; k < launches; ++k) {
+        const int upto = (int)((long long)nsteps * (k + 1) / launches);
+        const cudaError_t e = launch_chained(k_dns_steps<EX, EY, S, R, DIR>, grid, D::NT, k > 0, s, nf, a, psi,
+                                             b, cA, cD, upto - done, ul, ur);
+        if (e != cudaSuccess) return e;
+        done = upto;
+        std::swap(a, b);
+    }
+    if (a != u)
+        return cudaMemcpyAsync(u, a, (size_t)nf * nf * sizeof(float), cudaMemcpyDeviceToDevice, s);
+    return cudaGetLastError();
+}
+
+// Grids up to this side take several steps a launch: 1024^2 in 5.6 us a step against 8.2 for
+// k_dns_step<32>, the best of the others there; at 1536^2 that one takes 10.3 and the halo's
+// recomputation would cost about 12.
+constexpr int kDnsMultiMax = 1024;
+
 cudaError_t dns_run(int nf, float *u, float *u_tmp, const float *psi, double kappa, double dt,
                     int nsteps, cudaStream_t s)
 {
     const double h = 2.0 * kPi / nf;
     const float ax = (float)(1.0 / (2.0 * h));
     const float kd = (float)(kappa / (h * h));
+    if (nf <= kDnsMultiMax && !std::getenv("MLSD_DNS_TY")) {
+        g_dns_multi = true;
+        return dns_multi<false>(nf, u, u_tmp, psi, (float)dt * ax * ax, (float)dt * kd, nsteps, 0.f, 0.f, s);
+    }
+    g_dns_multi = false;
     // tensor maps of u, u_tmp and psi; boxes of DLX x (DTY + 4), one map set per tile height
     CUtensorMap m32[3], m64[3];
     const bool tma = encode_f32_2d(&m32[0], u, nf, nf, DLX, 36) &&
@@ -1063,6 +1243,7 @@ const char *dns_kernel_name()
     static const char *names[kDnsKinds] = {"k_dns_step<64>", "k_dns_step<32>", "k_dns_tma<32,1>",
                                            "k_dns_tma<32,2>", "k_dns_tma<64,1>",
                                            "k_dns_tma<32,1,pairs>"};
+    if (g_dns_multi) return "k_dns_steps";
     return g_dns_kind < 0 ? "" : names[g_dns_kind];
 }
 
@@ -1086,37 +1267,49 @@ cudaError_t launch_wait_check_tile(int *status, cudaStream_t s)
     return cudaGetLastError();
 }
 
-template <typename real>
-static cudaError_t dns_run_dirichlet_t(int nf, real *u, real *u_tmp, const float *psi,
-                                       double kappa, double dt, int nsteps, double ul, double ur,
-                                       cudaStream_t s)
+size_t dns_dirichlet_scratch_bytes(int nf, int precision, int nsteps)
 {
-    const double h = 2.0 * kPi / nf;
-    const real cA = (real)(dt / (4.0 * h * h));
-    const real cD = (real)(dt * kappa / (h * h));
-    const long long n2 = (long long)nf * nf;
-    const unsigned nb = (unsigned)((n2 + 255) / 256);
-    count_launches(1 + 2 * (long long)nsteps);
-    k_set_col0<real><<<(nf + 255) / 256, 256, 0, s>>>(nf, u, (real)ul);
-    for (int st = 0; st < nsteps; ++st) {
-        k_dns_dir_stage<false, real><<<nb, 256, 0, s>>>(nf, u, nullptr, psi, u_tmp, cA, cD,
-                                                        (real)ul, (real)ur);
-        // stage 2 writes u in place: each node reads only its own u
-        k_dns_dir_stage<true, real><<<nb, 256, 0, s>>>(nf, u, u_tmp, psi, u, cA, cD, (real)ul,
-                                                       (real)ur);
-    }
-    return cudaGetLastError();
+    return precision == MLSD_FP64 && nsteps > 0 ? 2 * (size_t)nf * nf * sizeof(double) : 0;
 }
 
 cudaError_t dns_run_dirichlet(int nf, void *u, void *u_tmp, const float *psi, int precision,
-                              double kappa, double dt, int nsteps, double ul, double ur,
+                              double kappa, double dt, int nsteps, double ul, double ur, void *scratch,
                               cudaStream_t s)
 {
-    if (precision == MLSD_FP64)
-        return dns_run_dirichlet_t<double>(nf, static_cast<double *>(u), static_cast<double *>(u_tmp),
-                                           psi, kappa, dt, nsteps, ul, ur, s);
-    return dns_run_dirichlet_t<float>(nf, static_cast<float *>(u), static_cast<float *>(u_tmp), psi,
-                                      kappa, dt, nsteps, ul, ur, s);
+    const double h = 2.0 * kPi / nf;
+    const double cA = dt / (4.0 * h * h), cD = dt * kappa / (h * h);
+    if (nsteps == 0) {
+        count_launches(1);
+        if (precision == MLSD_FP64)
+            k_set_col0<double><<<(nf + 255) / 256, 256, 0, s>>>(nf, static_cast<double *>(u), ul);
+        else
+            k_set_col0<float><<<(nf + 255) / 256, 256, 0, s>>>(nf, static_cast<float *>(u), (float)ul);
+        return cudaGetLastError();
+    }
+    if (precision != MLSD_FP64)
+        return dns_multi<true>(nf, static_cast<float *>(u), static_cast<float *>(u_tmp), psi, (float)cA,
+                               (float)cD, nsteps, (float)ul, (float)ur, s);
+    double *aE = static_cast<double *>(scratch), *aN = aE + (size_t)nf * nf;
+    const double r2 = 0.70710678118654752440;
+    const long long n2 = (long long)nf * nf;
+    count_launches(1 + (long long)nsteps);
+    k_dns_dir_coef<<<(unsigned)((n2 + 255) / 256), 256, 0, s>>>(nf, psi, r2 * cA, r2 * cD, aE, aN);
+    // tiles of 32 rows where they give every SM one, else of 8 (an SM's FP64 rate decides)
+    const unsigned gx = (unsigned)((nf + kD64TX - 1) / kD64TX);
+    const bool tall = (long long)gx * ((nf + 31) / 32) >= 152;
+    const int ty = tall ? 32 : 8, nt = 32 * (ty + 4) / kD64R;
+    const dim3 grid(gx, (unsigned)((nf + ty - 1) / ty));
+    const auto fn = tall ? k_dns_dir_step64<32> : k_dns_dir_step64<8>;
+    const double sq2 = 1.4142135623730951;
+    double *a = static_cast<double *>(u), *b = static_cast<double *>(u_tmp);
+    for (int k = 0; k < nsteps; ++k) {
+        const cudaError_t e = launch_chained(fn, grid, nt, k > 0, s, nf, a, b, aE, aN, r2 * cD, ul, ur,
+                                             sq2 * ul, sq2 * ur);
+        if (e != cudaSuccess) return e;
+        std::swap(a, b);
+    }
+    if (a != u) return cudaMemcpyAsync(u, a, (size_t)n2 * sizeof(double), cudaMemcpyDeviceToDevice, s);
+    return cudaGetLastError();
 }
 
 cudaError_t dns_vmax(int nf, const float *psi, unsigned *vmax_bits, cudaStream_t s)

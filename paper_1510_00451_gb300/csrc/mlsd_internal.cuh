@@ -166,8 +166,9 @@ cudaError_t macro_run_dirichlet(int N, void *U, int precision, const double *K, 
                                 int nsteps, double ul, double ur, double *mass_dev, void *scratch,
                                 cudaStream_t s);
 cudaError_t dns_run_dirichlet(int nf, void *u, void *u_tmp, const float *psi, int precision,
-                              double kappa, double dt, int nsteps, double ul, double ur,
+                              double kappa, double dt, int nsteps, double ul, double ur, void *scratch,
                               cudaStream_t s);
+size_t dns_dirichlet_scratch_bytes(int nf, int precision, int nsteps);
 size_t macro_scratch_bytes(int N, int precision, int nsteps);
 cudaError_t macro_dt_max(int N, const double *K, double *max_dev, cudaStream_t s);
 

@@ -1313,8 +1313,14 @@ int mlsd_dns_run_dirichlet(int nf, void *u_dev, void *u_tmp_dev, const float *ps
         !(dt > 0) || nsteps < 0 || !std::isfinite(u_left) || !std::isfinite(u_right))
         return MLSD_EINVAL;
     if (precision != MLSD_FP32 && precision != MLSD_FP64) return MLSD_EINVAL;
-    CK(dns_run_dirichlet(nf, u_dev, u_tmp_dev, psi_dev, precision, kappa, dt, nsteps, u_left,
-                         u_right, static_cast<cudaStream_t>(cuda_stream)));
+    cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+    const size_t sb = dns_dirichlet_scratch_bytes(nf, precision, nsteps);
+    void *scratch = nullptr;
+    if (sb) CK(cudaMallocAsync(&scratch, sb, s));
+    const cudaError_t e = dns_run_dirichlet(nf, u_dev, u_tmp_dev, psi_dev, precision, kappa, dt, nsteps,
+                                            u_left, u_right, scratch, s);
+    if (scratch) cudaFreeAsync(scratch, s);
+    CK(e);
     return MLSD_OK;
 }
 
