@@ -1378,6 +1378,281 @@ void add_variant_tm(std::vector<PatchVariant> &out)
 }
 
 // ---------------------------------------------------------------------------
+// FP64 patch solves, one CTA per field.  What bounds them is FP64 issue (2 operations a clock
+// and SM), so the step is written for the fewest of them; shared memory and registers have room
+// beside it.  With D the linear part of dt f and b its source (2 h A_J), Heun's step of this
+// affine problem is
+//   w <- w + D s + sigma,  s = w + D w / 2,  sigma = b + D b / 2,
+// and with D' = D / sqrt2 and s' = sqrt2 s both stages use the same coefficients:
+//   s' = c1 w + R(w),   w <- (w + sigma) + c2 s' + R(s'),
+//   R(x) = aE xE + aW xW + aN xN + aS xS + bx ((NE - NW) - (SE - SW)),
+//   aE, aW = (b11 +- A1) / sqrt2, aN, aS = (b22 +- A2) / sqrt2,
+//   c2 = -sqrt2 (b11 + b22), c1 = c2 + sqrt2.
+// aE and aN live in registers, aW, aS and sigma in shared memory.  With B12 = 0 (the finest
+// level of a chain without off-diagonal parts) the cross term is left out: x + 0 y = x.  In the
+// averaging window only the sum of w over the steps is kept per cell; the flux is linear in w,
+// so <v_i sum w> at the end is the sum of the <v_i w>.  Per cell-update that is 5 + 5 + 1
+// operations (8.5 + 8.5 + 1 with the cross term) and 1 in the window, against 10 + 11 and 3 in
+// the form before this one (Tile in FP64): the two-scale chain on 16^2 nodes, 2 x 256 patches
+// of 32^2 over the full window, 196 ms, 312 before.
+template <int N, int BX, int BY>
+struct Tile64 {
+    using T = Tile<N, 1, BX, BY, double>;
+    using S = Smem<N, 1, BX, BY, double>;
+    static constexpr int NBX = S::NBX, NBY = S::NBY, NT = NBX * NBY, CELLS = BX * BY;
+    // the window's sum of w: in registers for small blocks, else in shared memory
+    static constexpr bool WREG = CELLS <= 8;
+    // doubles: exchange (and set-up) buffers, reduction slots, then [CELLS][NT] arrays
+    static constexpr int RED = S::WORDS, ARR = RED + 64;
+    static constexpr int WORDS = ARR + (WREG ? 3 : 4) * CELLS * NT;
+    static constexpr size_t BYTES = (size_t)WORDS * sizeof(double);
+
+    struct Coef64 {
+        double c, b11x2, bx;                   // centre, 2 b11 / sqrt2, bx / sqrt2
+    };
+
+    // out = c x + R(x), plus out + sg when SECOND; x's edges go through buffer `buf`
+    template <bool CROSS, bool SECOND>
+    __device__ __forceinline__ static void stage(double *sm, int buf, int tx, int ty,
+                                                 const double (&x)[BY][BX], double (&out)[BY][BX],
+                                                 const double (&aE)[BY][BX], const double (&aN)[BY][BX],
+                                                 const double *aW, const double *aS, const double *sg,
+                                                 const Coef64 &k)
+    {
+        T::publish_edges(sm, buf, 0, tx, ty, x);
+        __syncthreads();
+        double hS[BX], hN[BX], hW[BY + 2], hE[BY + 2];
+        T::load_halos(sm, buf, tx, ty, hS, hN, hW, hE);
+        double dm[BX], d0[BX], dp[BX];
+        if constexpr (CROSS) {
+            T::halo_diff(dm, hS, 0, hW, hE);
+            T::row_diff(d0, x, 0, hW, hE);
+        }
+#pragma unroll
+        for (int r = 0; r < BY; ++r) {
+            if constexpr (CROSS) {
+                if (r + 1 < BY) T::row_diff(dp, x, (r + 1) % BY, hW, hE);
+                else T::halo_diff(dp, hN, BY + 1, hW, hE);
+            }
+#pragma unroll
+            for (int c = 0; c < BX; ++c) {
+                const int i = (r * BX + c) * NT;
+                const double xE = c + 1 < BX ? x[r][(c + 1) % BX] : hE[r + 1];
+                const double xW = c > 0 ? x[r][(c + BX - 1) % BX] : hW[r + 1];
+                const double xN = r + 1 < BY ? x[(r + 1) % BY][c] : hN[c];
+                const double xS = r > 0 ? x[(r + BY - 1) % BY][c] : hS[c];
+                double g = SECOND ? fma(k.c, x[r][c], out[r][c] + sg[i]) : k.c * x[r][c];
+                if constexpr (CROSS) {
+                    // aE (xE - xW) + 2 b11 xW = aE xE + aW xW, the difference being there already
+                    g = fma(aE[r][c], d0[c], g);
+                    g = fma(k.b11x2, xW, g);
+                    g = fma(k.bx, dp[c] - dm[c], g);
+                } else {
+                    g = fma(aE[r][c], xE, g);
+                    g = fma(aW[i], xW, g);
+                }
+                g = fma(aN[r][c], xN, g);
+                out[r][c] = fma(aS[i], xS, g);
+            }
+            if constexpr (CROSS) {
+#pragma unroll
+                for (int c = 0; c < BX; ++c) { dm[c] = d0[c]; d0[c] = dp[c]; }
+            }
+        }
+    }
+
+    template <int J, bool CROSS>
+    __device__ static void steps(const PatchParams &prm, double *sm, long long p, int tx, int ty,
+                                 const double (&aE)[BY][BX], const double (&aN)[BY][BX], double *arr,
+                                 double c1, double c2, double b11l, double b22l, double bxl, long long nb,
+                                 long long na, double &f1, double &f2)
+    {
+        const int tid = threadIdx.x, a0 = tx * BX, b0 = ty * BY;
+        double *aW = arr + tid, *aS = aW + CELLS * NT, *sg = aS + CELLS * NT, *wsm = sg + CELLS * NT;
+        Coef64 k;
+        k.b11x2 = 2.0 * b11l;
+        k.bx = bxl;
+        double w[BY][BX], s[BY][BX], ws[WREG ? CELLS : 1];
+        // sigma = b + D b / 2 = b + D' b / sqrt2, b held in sg on entry
+#pragma unroll
+        for (int r = 0; r < BY; ++r)
+#pragma unroll
+            for (int c = 0; c < BX; ++c) w[r][c] = sg[(r * BX + c) * NT];
+        k.c = c2;
+        stage<CROSS, false>(sm, 0, tx, ty, w, s, aE, aN, aW, aS, sg, k);
+#pragma unroll
+        for (int r = 0; r < BY; ++r)
+#pragma unroll
+            for (int c = 0; c < BX; ++c) {
+                const int i = r * BX + c;
+                sg[i * NT] = fma(0.70710678118654752440, s[r][c], w[r][c]);
+                w[r][c] = 0.0;
+                if constexpr (WREG) ws[i] = 0.0;
+                else wsm[i * NT] = 0.0;
+            }
+        __syncthreads();                       // buffer 0 is read before it is written again
+        const long long ntot = nb + na;
+        for (long long step = 0; step < ntot; ++step) {
+            k.c = c1;
+            stage<CROSS, false>(sm, 0, tx, ty, w, s, aE, aN, aW, aS, sg, k);
+            k.c = c2;
+            stage<CROSS, true>(sm, 1, tx, ty, s, w, aE, aN, aW, aS, sg, k);
+            if (step >= nb) {
+#pragma unroll
+                for (int r = 0; r < BY; ++r)
+#pragma unroll
+                    for (int c = 0; c < BX; ++c) {
+                        const int i = r * BX + c;
+                        if constexpr (WREG) ws[i] += w[r][c];
+                        else wsm[i * NT] += w[r][c];
+                    }
+            }
+        }
+        // sqrt2 sum (A_i) (window sum of w), A_1 / sqrt2 = aE - b11 / sqrt2
+#pragma unroll
+        for (int r = 0; r < BY; ++r)
+#pragma unroll
+            for (int c = 0; c < BX; ++c) {
+                const int i = r * BX + c;
+                const double v = WREG ? ws[WREG ? i : 0] : wsm[i * NT];
+                f1 = fma(aE[r][c] - b11l, v, f1);
+                f2 = fma(aN[r][c] - b22l, v, f2);
+            }
+        f1 *= 1.41421356237309504880;
+        f2 *= 1.41421356237309504880;
+        if (prm.wdump) {
+            double *wd = static_cast<double *>(prm.wdump) + (2 * p + (J - 1)) * (long long)N * N;
+#pragma unroll
+            for (int r = 0; r < BY; ++r)
+#pragma unroll
+                for (int c = 0; c < BX; ++c) wd[(b0 + r) * N + a0 + c] = w[r][c];
+        }
+    }
+
+    template <int J>
+    __device__ static void run(const PatchParams &prm, double *sm, long long p)
+    {
+        const int tid = threadIdx.x, tx = tid % NBX, ty = tid / NBX;
+        const int a0 = tx * BX, b0 = ty * BY;
+        double *red = sm + RED, *arr = sm + ARR;
+        const long long Nl = prm.Nl;
+        const long long ox = patch_origin(p % prm.n_macro, prm.n_macro, Nl, N);
+        const long long oy = patch_origin(p / prm.n_macro, prm.n_macro, Nl, N);
+        // ---- set-up as Tile::run: psi, velocity, time step ----
+        double *psi = sm;
+        const double *band = static_cast<const double *>(prm.band);
+        for (int c = tid; c < N * N; c += NT) psi[c] = patch_band(band, Nl, prm.tile, p, ox, oy, N, c % N, c / N);
+        __syncthreads();
+        const double inv2h = 1.0 / (2.0 * prm.h);
+        double aE[BY][BX], aN[BY][BX];
+        double vmax = 0;
+#pragma unroll
+        for (int r = 0; r < BY; ++r) {
+            const int b = b0 + r, bp = (b + 1) % N, bm = (b + N - 1) % N;
+#pragma unroll
+            for (int c = 0; c < BX; ++c) {
+                const int a = a0 + c, ap = (a + 1) % N, am = (a + N - 1) % N;
+                aE[r][c] = (psi[bm * N + a] - psi[bp * N + a]) * inv2h;
+                aN[r][c] = (psi[b * N + ap] - psi[b * N + am]) * inv2h;
+                vmax = fmax(vmax, fabs(aE[r][c]) + fabs(aN[r][c]));
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) vmax = fmax(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
+        if ((tid & 31) == 0) red[tid >> 5] = vmax;
+        __syncthreads();
+        double vm = 0.0;
+        for (int k = 0; k < NT / 32; ++k) vm = fmax(vm, red[k]);
+        const double B11 = prm.Kb[3 * p], B12 = prm.Kb[3 * p + 1], B22 = prm.Kb[3 * p + 2];
+        double dt;
+        long long nb, na;
+        micro_schedule(prm.h, prm.L, vm, B11, B12, B22, prm.cfl, prm.t_burn, prm.t_avg,
+                       prm.nb_fixed, prm.na_fixed, dt, nb, na);
+        if (!(dt > 0.0) || !isfinite(dt) || nb < 0 || na < 1 || nb + na > kMaxSteps) {
+            if (tid == 0) {
+                prm.S[4 * p + 2 * (J - 1)] = __longlong_as_double(0x7ff8000000000000ll);
+                prm.S[4 * p + 2 * (J - 1) + 1] = __longlong_as_double(0x7ff8000000000000ll);
+                atomicCAS(prm.status, 0, MLSD_EINVAL);
+            }
+            return;
+        }
+        if (J == 1 && tid == 0 && prm.steps) { prm.steps[p] = nb + na; prm.steps[prm.P + p] = na; }
+        const double r2 = 0.70710678118654752440, hh = prm.h * prm.h;
+        const double cA = dt / (2.0 * prm.h);
+        const double b11 = dt * B11 / hh, b22 = dt * B22 / hh, b11l = r2 * b11, b22l = r2 * b22;
+        const double bxl = r2 * (dt * B12 / (2.0 * hh));
+        const double c2 = -2.0 * (b11l + b22l), c1 = 1.41421356237309504880 + c2;
+#pragma unroll
+        for (int r = 0; r < BY; ++r)
+#pragma unroll
+            for (int c = 0; c < BX; ++c) {
+                const int i = (r * BX + c) * NT + tid;
+                const double A1 = aE[r][c] * cA, A2 = aN[r][c] * cA;
+                aE[r][c] = fma(r2, A1, b11l);
+                aN[r][c] = fma(r2, A2, b22l);
+                arr[i] = fma(-r2, A1, b11l);
+                arr[CELLS * NT + i] = fma(-r2, A2, b22l);
+                arr[2 * CELLS * NT + i] = 2.0 * prm.h * (J == 1 ? A1 : A2);
+            }
+        __syncthreads();                       // psi and the vmax slots are dead
+        double f1 = 0.0, f2 = 0.0;
+        if (B12 != 0.0)
+            steps<J, true>(prm, sm, p, tx, ty, aE, aN, arr, c1, c2, b11l, b22l, bxl, nb, na, f1, f2);
+        else
+            steps<J, false>(prm, sm, p, tx, ty, aE, aN, arr, c1, c2, b11l, b22l, bxl, nb, na, f1, f2);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            f1 += __shfl_xor_sync(0xffffffffu, f1, o);
+            f2 += __shfl_xor_sync(0xffffffffu, f2, o);
+        }
+        __syncthreads();
+        if ((tid & 31) == 0) { red[2 * (tid >> 5)] = f1; red[2 * (tid >> 5) + 1] = f2; }
+        __syncthreads();
+        if (tid == 0) {
+            double t1 = 0.0, t2 = 0.0;
+            for (int k = 0; k < NT / 32; ++k) { t1 += red[2 * k]; t2 += red[2 * k + 1]; }
+            const double scale = 1.0 / (cA * (double)N * (double)N * (double)na);
+            const double s1j = t1 * scale, s2j = t2 * scale;
+            prm.S[4 * p + 2 * (J - 1)] = s1j;
+            prm.S[4 * p + 2 * (J - 1) + 1] = s2j;
+            if (!isfinite(s1j) || !isfinite(s2j)) atomicCAS(prm.status, 0, MLSD_ENONFINITE);
+        }
+    }
+};
+
+template <int N, int BX, int BY>
+__global__ void __launch_bounds__((N / BX) * (N / BY)) k_patch_solve64(PatchParams prm)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double *sm = reinterpret_cast<double *>(smem_raw);
+    const long long item = prm.item0 + blockIdx.x;
+    if (item >= prm.item0 + prm.items) return;
+    const long long p = prm.pidx ? (long long)prm.pidx[item >> 1] : (item >> 1);
+    if (item & 1) Tile64<N, BX, BY>::template run<2>(prm, sm, p);
+    else Tile64<N, BX, BY>::template run<1>(prm, sm, p);
+}
+
+template <int N, int BX, int BY>
+void add_variant64(std::vector<PatchVariant> &out)
+{
+    static_assert(((N / BX) * (N / BY)) % 32 == 0 && (N / BX) * (N / BY) <= 1024, "whole warps only");
+    PatchVariant v;
+    v.n = N;
+    v.precision = MLSD_FP64;
+    v.bx = BX;
+    v.by = BY;
+    v.minb = 1;
+    v.packed = 0;
+    v.cluster = 1;
+    v.split = 0;
+    v.tmem = 0;
+    v.threads = (N / BX) * (N / BY);
+    v.smem = Tile64<N, BX, BY>::BYTES;
+    v.fn = reinterpret_cast<const void *>(&k_patch_solve64<N, BX, BY>);
+    out.push_back(v);
+}
+
+// ---------------------------------------------------------------------------
 // Packed variant: one CTA advances BOTH corrector fields of a patch, each cell
 // holding (w_1, w_2) in one float2 and every stencil operation issued as a
 // Blackwell f32x2 instruction (FFMA2 / FADD2 / FMUL2).  The two fields share

@@ -17,8 +17,8 @@ int patch_variants_n32(int precision, std::vector<PatchVariant> &out)
         add_variant2<32, 2, 4>(out);
         add_variant2<32, 4, 2>(out);
     } else {
-        add_variant<32, 2, 4, double>(out);
-        add_variant<32, 4, 4, double>(out);
+        add_variant64<32, 2, 4>(out);
+        add_variant64<32, 4, 4>(out);
     }
     return (int)out.size();
 }
