@@ -48,3 +48,23 @@ def test_macro_edges(mlsd, torch_mod, N, steps, prec):
     Wr = oracle.macro_run_dirichlet(U0, K, dt, steps, 1.25, -0.5)
     assert torch_mod.all(W[:, 0] == 1.25)
     assert rel_l2(W.cpu().numpy(), Wr) < tol
+
+
+@pytest.mark.parametrize("n,tile", [(32, "4x4"), (32, "2x4"), (32, "4x4p"), (64, "4x8m3"), (64, "4x4p")])
+def test_no_cross_term_is_the_same(mlsd, torch_mod, monkeypatch, n, tile):
+    # B12 = 0 leaves the cross term out; a B12 so small that its products vanish against
+    # every sum keeps it and has to give the same bits
+    monkeypatch.setenv("MLSD_TILE", tile)
+    lv = mlsd.Levels(flows.cellular_two_scale(0.8, 0.5, 4), 0.03, 3, [1, 4, 8], [n, n],
+                     n_burn_fixed=40, n_avg_fixed=35)
+    B = random_spd(9, np.random.default_rng(n), 0.03, 0.1)
+    out = []
+    for b12 in (0.0, 1e-30):
+        B[:, 1] = b12
+        Kb = torch_mod.tensor(B, dtype=torch_mod.float64, device="cuda:0")
+        K, w = torch_mod.zeros_like(Kb), torch_mod.zeros(9, 2, n, n, device="cuda:0")
+        lv.solve_level(2, Kb, K, w)
+        assert lv.status() == 0
+        out.append((K, w))
+    assert torch_mod.equal(out[0][1], out[1][1])
+    assert torch_mod.equal(out[0][0][:, ::2], out[1][0][:, ::2])
