@@ -110,6 +110,53 @@ struct mlsd_levels {
 
 namespace {
 
+// Stream-ordered workspaces of single calls.  The device's default pool gives its memory back to
+// the system at every synchronisation, and the next call maps it again (about 150 us a call);
+// the library's own pool, one per device, keeps up to kPoolKeep bytes.  mlsd_free_levels and
+// mlsd_surrogate_free give back what is idle.  The pool itself orders allocations and frees
+// between streams and threads.
+constexpr unsigned long long kPoolKeep = 32ull << 20;
+std::mutex g_pool_mu;
+std::map<int, cudaMemPool_t> g_pool;
+
+cudaError_t ws_alloc(void **p, size_t bytes, cudaStream_t s)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    cudaMemPool_t pool = nullptr;
+    {
+        std::lock_guard<std::mutex> lock(g_pool_mu);
+        auto it = g_pool.find(dev);
+        if (it == g_pool.end()) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.handleTypes = cudaMemHandleTypeNone;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            unsigned long long keep = kPoolKeep;
+            if ((e = cudaMemPoolCreate(&pool, &props)) != cudaSuccess) return e;
+            if ((e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+                cudaMemPoolDestroy(pool);
+                return e;
+            }
+            it = g_pool.emplace(dev, pool).first;
+        }
+        pool = it->second;
+    }
+    return cudaMallocFromPoolAsync(p, bytes, pool, s);
+}
+
+// give back the idle memory of the current device's pool (after a device synchronisation)
+void ws_trim()
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    auto it = g_pool.find(dev);
+    if (it != g_pool.end()) cudaMemPoolTrimTo(it->second, 0);
+}
+
 int dev_alloc(mlsd_levels *h, void **p, size_t bytes)
 {
     *p = nullptr;
@@ -855,6 +902,7 @@ void mlsd_free_levels(mlsd_levels *h)
     if (h->graph_sur) cudaGraphExecDestroy(h->graph_sur);
     if (h->cap) cudaStreamDestroy(h->cap);
     for (void *p : h->allocs) cudaFree(p);
+    ws_trim();
     delete h;
 }
 
@@ -1204,7 +1252,7 @@ int mlsd_macro_step(int n_macro, void *U_dev, int precision, const double *K_dev
     const size_t sb = macro_scratch_bytes(n_macro, precision, nsteps);
     const size_t mb = mass_out_host ? (size_t)(nsteps + 1) * sizeof(double) : 0;
     void *scratch = nullptr;
-    if (sb + mb) CK(cudaMallocAsync(&scratch, sb + mb + 256, s));
+    if (sb + mb) CK(ws_alloc(&scratch, sb + mb + 256, s));
     double *mass = mass_out_host
         ? reinterpret_cast<double *>((reinterpret_cast<uintptr_t>(scratch) + sb + 255) & ~(uintptr_t)255)
         : nullptr;
@@ -1228,7 +1276,7 @@ int mlsd_macro_step_dirichlet(int n_macro, void *U_dev, int precision, const dou
     const size_t sb = macro_scratch_bytes(n_macro, precision, nsteps);
     const size_t mb = mass_out_host ? (size_t)(nsteps + 1) * sizeof(double) : 0;
     void *scratch = nullptr;
-    if (sb + mb) CK(cudaMallocAsync(&scratch, sb + mb + 256, s));
+    if (sb + mb) CK(ws_alloc(&scratch, sb + mb + 256, s));
     double *mass = mass_out_host
         ? reinterpret_cast<double *>((reinterpret_cast<uintptr_t>(scratch) + sb + 255) & ~(uintptr_t)255)
         : nullptr;
@@ -1248,7 +1296,7 @@ int mlsd_macro_dt(int n_macro, const double *K_dev, double cfl, double *dt_out_h
     if (n_macro < 2 || !K_dev || !(cfl > 0) || !dt_out_host) return MLSD_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     double *m = nullptr;
-    CK(cudaMallocAsync((void **)&m, sizeof(double), s));
+    CK(ws_alloc((void **)&m, sizeof(double), s));
     cudaError_t e = macro_dt_max(n_macro, K_dev, m, s);
     double mx = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&mx, m, sizeof(double), cudaMemcpyDeviceToHost, s);
@@ -1274,7 +1322,7 @@ int mlsd_grid_psi(int n_modes, const int32_t *k1, const int32_t *k2, const doubl
     const size_t mb = (pk.blob.size() + 255) / 256 * 256;
     const size_t gb = (pk.groups + 1) * (size_t)nf * sizeof(double2);
     char *ws = nullptr;
-    CK(cudaMallocAsync((void **)&ws, mb + gb, s));
+    CK(ws_alloc((void **)&ws, mb + gb, s));
     cudaError_t e = cudaMemcpyAsync(ws, pk.blob.data(), pk.blob.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
         e = launch_band_synth(pk.at(ws), nf, reinterpret_cast<double2 *>(ws + mb), psi_dev, 0, s);
@@ -1316,7 +1364,7 @@ int mlsd_dns_run_dirichlet(int nf, void *u_dev, void *u_tmp_dev, const float *ps
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     const size_t sb = dns_dirichlet_scratch_bytes(nf, precision, nsteps);
     void *scratch = nullptr;
-    if (sb) CK(cudaMallocAsync(&scratch, sb, s));
+    if (sb) CK(ws_alloc(&scratch, sb, s));
     const cudaError_t e = dns_run_dirichlet(nf, u_dev, u_tmp_dev, psi_dev, precision, kappa, dt, nsteps,
                                             u_left, u_right, scratch, s);
     if (scratch) cudaFreeAsync(scratch, s);
@@ -1330,7 +1378,7 @@ int mlsd_dns_dt(int nf, const float *psi_dev, double kappa, double cfl, double *
     if (nf < 2 || !psi_dev || !(kappa > 0) || !(cfl > 0) || !dt_out_host) return MLSD_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     unsigned *m = nullptr;
-    CK(cudaMallocAsync((void **)&m, sizeof(unsigned), s));
+    CK(ws_alloc((void **)&m, sizeof(unsigned), s));
     cudaError_t e = dns_vmax(nf, psi_dev, m, s);
     unsigned bits = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&bits, m, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
@@ -1354,7 +1402,7 @@ int mlsd_coarse_grain(int nf, const float *u_dev, int n_macro, float *U_dev,
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     double *m = nullptr;
     if (mass_out_host)
-        CK(cudaMallocAsync((void **)&m, (1 + (size_t)n_macro * n_macro) * sizeof(double), s));
+        CK(ws_alloc((void **)&m, (1 + (size_t)n_macro * n_macro) * sizeof(double), s));
     cudaError_t e = coarse_grain(nf, u_dev, n_macro, U_dev, m, s);
     if (e == cudaSuccess && m) e = cudaMemcpyAsync(mass_out_host, m, sizeof(double), cudaMemcpyDeviceToHost, s);
     if (m) cudaFreeAsync(m, s);
@@ -1422,6 +1470,7 @@ void mlsd_surrogate_free(mlsd_surrogate *s)
     if (!s) return;
     cudaDeviceSynchronize();
     for (void *p : s->allocs) cudaFree(p);
+    ws_trim();
     delete s;
 }
 
@@ -1573,7 +1622,7 @@ int mlsd_surrogate_dataset(mlsd_levels *h, int level, const double *B_dev, void 
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const long long P = h->P;
     double *ws = nullptr;
-    CK(cudaMallocAsync((void **)&ws, (size_t)P * 7 * 8, st));
+    CK(ws_alloc((void **)&ws, (size_t)P * 7 * 8, st));
     double *K = ws, *Q = ws + 3 * P;                 // Q: E and the series gap, [P][4]
     int rc = mlsd_solve_level(h, level, B_dev, K, nullptr, cuda_stream);
     cudaError_t e = cudaSuccess;
@@ -1621,7 +1670,7 @@ int mlsd_surrogate_train(mlsd_surrogate *s, const void *X_dev, const float *Y_de
     const long long steps = rows / batch, total = steps * epochs;
     char *ws = nullptr;
     const size_t xb = (size_t)batch * MLSD_SUR_IN * 2, yb = (size_t)batch * 3 * 4, ib = (size_t)rows * 4;
-    CK(cudaMallocAsync((void **)&ws, xb + yb + ib + 16, st));
+    CK(ws_alloc((void **)&ws, xb + yb + ib + 16, st));
     void *Xb = ws;
     float *Yb = reinterpret_cast<float *>(ws + xb);
     int *idx = reinterpret_cast<int *>(ws + xb + yb);
@@ -1755,7 +1804,7 @@ int mlsd_solve_level_surrogate(mlsd_levels *h, mlsd_surrogate *s, int level,
     char *ws = nullptr;
     const size_t xb = (size_t)P * MLSD_SUR_IN * 2, ob = (size_t)s->members * P * 3 * 4;
     const size_t fb = (size_t)P * 4, ib = (size_t)P * 4, qb = (size_t)P * 4 * 8;
-    CK(cudaMallocAsync((void **)&ws, qb + xb + ob + fb + ib + 256, st));
+    CK(ws_alloc((void **)&ws, qb + xb + ob + fb + ib + 256, st));
     double *Q = reinterpret_cast<double *>(ws);
     void *X = ws + qb;
     float *out = reinterpret_cast<float *>(ws + qb + xb);
