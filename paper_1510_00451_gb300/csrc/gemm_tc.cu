@@ -45,9 +45,12 @@ struct GtArgs {
     const float *Zprev;                    // backward: [M][N]
     __nv_bfloat16 *out, *outT;             // forward act / backward dZ: [M][N] and [N][ldT]
     int ldT;
-    float *part;                           // partial: [gridDim.z][M][N]
+    float *part;                           // partial: [slices][M][N]
+    int slices;                            // K slices of this problem (gridDim.z of it)
     int *status;
 };
+// NP problems in one launch: blockIdx.z runs over the slices of all of them
+template <int NP> struct GtBatch { GtArgs p[NP]; };
 
 __device__ __forceinline__ uint32_t s_u32(const void *p)
 {
@@ -106,9 +109,17 @@ __device__ __forceinline__ float gt_gelu_d(float z)
     return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
 }
 
-template <int BN>
-__global__ void __launch_bounds__(GT_THREADS, 1) k_gemm_tc(const __grid_constant__ GtArgs a)
+template <int BN, int NP>
+__global__ void __launch_bounds__(GT_THREADS, 1) k_gemm_tc(const __grid_constant__ GtBatch<NP> batch)
 {
+    int prob = 0, slice = blockIdx.z;
+    if constexpr (NP > 1)
+        while (prob + 1 < NP && slice >= batch.p[prob].slices) slice -= batch.p[prob++].slices;
+    const GtArgs &a = batch.p[prob];
+    if ((int)blockIdx.x * BN >= a.N || (int)blockIdx.y * GT_M >= a.M) {      // a smaller problem's edge
+        chain_wait();
+        return;
+    }
     constexpr int A_BYTES = GT_M * GT_KC * 2, B_BYTES = BN * GT_KC * 2, SLOT = A_BYTES + B_BYTES;
     constexpr int GT_RING = gt_ring<BN>();
     constexpr uint32_t TCOLS = BN <= 32 ? 32 : (BN <= 64 ? 64 : (BN <= 128 ? 128 : 256));
@@ -119,7 +130,7 @@ __global__ void __launch_bounds__(GT_THREADS, 1) k_gemm_tc(const __grid_constant
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.y * GT_M, n0 = blockIdx.x * BN;
     const int kc_total = (a.K + GT_KC - 1) / GT_KC;
-    const int kc0 = blockIdx.z * a.kc_slice;
+    const int kc0 = slice * a.kc_slice;
     const int nk = max(0, min(a.kc_slice, kc_total - kc0));
     const CUtensorMap *pa = &a.amap, *pb = &a.bmap;
 
@@ -142,6 +153,7 @@ __global__ void __launch_bounds__(GT_THREADS, 1) k_gemm_tc(const __grid_constant
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
+    chain_wait();
 
     auto issue = [&](int q) {
         const int slot = q % GT_RING;
@@ -231,7 +243,7 @@ __global__ void __launch_bounds__(GT_THREADS, 1) k_gemm_tc(const __grid_constant
             const int nb = n0 + c0;
             if (a.mode == GT_PART) {
                 if (m < a.M) {
-                    float *dst = a.part + ((long long)blockIdx.z * a.M + m) * a.N + nb;
+                    float *dst = a.part + ((long long)slice * a.M + m) * a.N + nb;
 #pragma unroll
                     for (int i = 0; i < 32; i += 4)
                         *reinterpret_cast<float4 *>(dst + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
@@ -291,21 +303,33 @@ __global__ void __launch_bounds__(GT_THREADS, 1) k_gemm_tc(const __grid_constant
     }
 }
 
-template <int BN>
-cudaError_t launch_gt(const GtArgs &a, int splits, cudaStream_t s)
+template <int BN, int NP>
+cudaError_t launch_gt(const GtBatch<NP> &b, bool overlap, cudaStream_t s)
 {
     constexpr size_t smem = (size_t)gt_ring<BN>() * (GT_M * GT_KC * 2 + BN * GT_KC * 2);
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&k_gemm_tc<BN>),
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
-    dim3 g((unsigned)((a.N + BN - 1) / BN), (unsigned)((a.M + GT_M - 1) / GT_M), (unsigned)splits);
+    const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&k_gemm_tc<BN, NP>),
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int M = 0, N = 0, z = 0;
+    for (const GtArgs &a : b.p) { M = std::max(M, a.M); N = std::max(N, a.N); z += a.slices; }
+    const dim3 g((unsigned)((N + BN - 1) / BN), (unsigned)((M + GT_M - 1) / GT_M), (unsigned)z);
     count_launches(1);
-    k_gemm_tc<BN><<<g, GT_THREADS, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_gemm_tc<BN, NP>, g, GT_THREADS, smem, overlap, s, b);
+}
+
+// tensor maps and slicing of one problem for BN-column tiles
+bool fill_gt(GtArgs &a, int bn, int mode, int M, int N, int K, const void *A, long long lda, const void *B,
+             long long ldb, int splits)
+{
+    if (!encode_rows_bf16(&a.amap, A, M, K, lda, GT_M) || !encode_rows_bf16(&a.bmap, B, N, K, ldb, bn))
+        return false;
+    a.M = M; a.N = N; a.K = K;
+    a.mode = mode;
+    const int kc_total = (K + GT_KC - 1) / GT_KC;
+    splits = std::min(splits, kc_total);
+    a.kc_slice = (kc_total + splits - 1) / splits;
+    a.slices = (kc_total + a.kc_slice - 1) / a.kc_slice;     // no empty slice
+    return true;
 }
 
 }  // namespace
@@ -313,18 +337,15 @@ cudaError_t launch_gt(const GtArgs &a, int splits, cudaStream_t s)
 // One tensor-core GEMM (see the top of the file).  A: M rows of K bfloat16
 // elements, lda apart; B: N rows of K, ldb apart (lda, ldb multiples of 8, both at
 // least K rounded up to 8, their padding zero).  mode 0 forward (bias, Z, act,
-// actT), 1 backward (Zprev, dZ, dZT), 2 partial sums of up to `splits` K slices
-// into part [slices][M][N], the number of slices used returned in *slices.  In the
-// forward mode Z and the transpose may be NULL.
+// actT), 1 backward (Zprev, dZ, dZT).  In the forward mode Z and the transpose may be NULL.
+// overlap: the launch is part of a chain (launch_chained).
 // BN = 128, or 64 where 128-column tiles would fill less than a third of the SMs
 // (256 with MLSD_GEMM_BN=256 where N is a multiple of 256).
 cudaError_t gemm_tc(int mode, int M, int N, int K, const void *A, long long lda, const void *B,
                     long long ldb, const float *bias, float *Z, const float *Zprev, void *out,
-                    void *outT, int ldT, float *part, int splits, int *slices, int *status,
-                    cudaStream_t s)
+                    void *outT, int ldT, int *status, bool overlap, cudaStream_t s)
 {
-    if (M < 1 || N < 1 || K < 1 || splits < 1 || N % 32) return cudaErrorInvalidValue;
-    if (mode != GT_PART) splits = 1;
+    if (M < 1 || N < 1 || K < 1 || N % 32 || mode == GT_PART) return cudaErrorInvalidValue;
     // 128-column tiles: twice the CTAs of 256-column ones on these short GEMMs
     // (MLSD_GEMM_BN=256 selects the wide tile where N is a multiple of 256)
     static const bool wide = [] { const char *e = std::getenv("MLSD_GEMM_BN"); return e && std::atoi(e) == 256; }();
@@ -333,27 +354,35 @@ cudaError_t gemm_tc(int mode, int M, int N, int K, const void *A, long long lda,
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         sms = 152;
-    const long long tiles128 = (long long)((N + 127) / 128) * ((M + GT_M - 1) / GT_M) * splits;
+    const long long tiles128 = (long long)((N + 127) / 128) * ((M + GT_M - 1) / GT_M);
     const int bn = (wide && N % 256 == 0) ? 256 : (tiles128 * 3 < sms ? 64 : 128);
-    GtArgs a;
-    if (!encode_rows_bf16(&a.amap, A, M, K, lda, GT_M) ||
-        !encode_rows_bf16(&a.bmap, B, N, K, ldb, bn))
-        return cudaErrorNotSupported;
-    a.M = M; a.N = N; a.K = K;
-    const int kc_total = (K + GT_KC - 1) / GT_KC;
-    splits = std::min(splits, kc_total);
-    a.kc_slice = (kc_total + splits - 1) / splits;
-    splits = (kc_total + a.kc_slice - 1) / a.kc_slice;       // no empty slice
-    a.mode = mode;
+    GtBatch<1> b = {};
+    GtArgs &a = b.p[0];
+    if (!fill_gt(a, bn, mode, M, N, K, A, lda, B, ldb, 1)) return cudaErrorNotSupported;
     a.bias = bias; a.Z = Z; a.Zprev = Zprev;
     a.out = static_cast<__nv_bfloat16 *>(out);
     a.outT = static_cast<__nv_bfloat16 *>(outT);
     a.ldT = ldT;
-    a.part = part;
     a.status = status;
-    if (slices) *slices = splits;
-    return bn == 256 ? launch_gt<256>(a, splits, s)
-                     : (bn == 128 ? launch_gt<128>(a, splits, s) : launch_gt<64>(a, splits, s));
+    return bn == 256 ? launch_gt<256, 1>(b, overlap, s)
+                     : (bn == 128 ? launch_gt<128, 1>(b, overlap, s) : launch_gt<64, 1>(b, overlap, s));
+}
+
+// Three GEMMs D = A B^T in one launch, each the partial sums of up to g.splits K slices into
+// g.part [slices][M][N]; g.splits becomes the number of slices used.  The tiles of one of them
+// alone would leave most SMs idle.
+cudaError_t gemm_tc_parts(GemmPart (&g)[3], int *status, bool overlap, cudaStream_t s)
+{
+    GtBatch<3> b = {};
+    for (int i = 0; i < 3; ++i) {
+        if (g[i].M < 1 || g[i].N < 1 || g[i].K < 1 || g[i].splits < 1 || g[i].N % 32) return cudaErrorInvalidValue;
+        if (!fill_gt(b.p[i], 64, GT_PART, g[i].M, g[i].N, g[i].K, g[i].A, g[i].lda, g[i].B, g[i].ldb, g[i].splits))
+            return cudaErrorNotSupported;
+        b.p[i].part = g[i].part;
+        b.p[i].status = status;
+        g[i].splits = b.p[i].slices;
+    }
+    return launch_gt<64, 3>(b, overlap, s);
 }
 
 int gemm_tc_splits(int M, int N, int K, int sms)

@@ -27,16 +27,6 @@
 namespace mlsd {
 namespace {
 
-// Chains of launches that each read what the one before wrote: a kernel launched with
-// launch_chained starts while its predecessor still runs, loads what the predecessor does not
-// write (coefficients), and calls chain_wait before it reads or writes the fields.
-// The successor is let in only after that wait: one launch ahead, no further.
-__device__ __forceinline__ void chain_wait()
-{
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 // deterministic FP64 block sum (all threads return the total)
 __device__ double block_sum(double v, double *red)
 {
@@ -941,23 +931,6 @@ static long long macro_mass_blocks(int N, int precision)
     return std::max(((long long)N * N + 255) / 256, macro_tiles(N, precision));
 }
 
-// launch a kernel of a chain; overlap: let it start before its predecessor in the stream ends
-template <typename... P, typename... A>
-static cudaError_t launch_chained(void (*fn)(P...), dim3 grid, int threads, bool overlap, cudaStream_t s,
-                                  A... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = overlap ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, fn, P(args)...);
-}
-
 size_t macro_scratch_bytes(int N, int precision, int nsteps)
 {
     const size_t rs = precision == MLSD_FP64 ? 8 : 4;
@@ -999,7 +972,7 @@ static cudaError_t macro_run_t(int N, real *U, const double *K, double dt, int n
     real *a = start_in_V ? V : U, *b = start_in_V ? U : V;
     for (int k = 0; k < nsteps; k += S) {
         const cudaError_t e = launch_chained(
-            k_macro_tile<real, kTileX, TY, S, DIR>, grid, (T::NT + 31) / 32 * 32, k > 0, s, N, a, b, co,
+            k_macro_tile<real, kTileX, TY, S, DIR>, grid, (T::NT + 31) / 32 * 32, 0, k > 0, s, N, a, b, co,
             std::min(S, nsteps - k), mass ? part + stride + (size_t)k * tiles : nullptr, r);
         if (e != cudaSuccess) return e;
         std::swap(a, b);
@@ -1156,7 +1129,7 @@ static cudaError_t dns_multi(int nf, float *u, float *u_tmp, const float *psi, f
     float *a = u, *b = u_tmp;
     for (int k = 0, done = 0; k < launches; ++k) {
         const int upto = (int)((long long)nsteps * (k + 1) / launches);
-        const cudaError_t e = launch_chained(k_dns_steps<EX, EY, S, R, DIR>, grid, D::NT, k > 0, s, nf, a, psi,
+        const cudaError_t e = launch_chained(k_dns_steps<EX, EY, S, R, DIR>, grid, D::NT, 0, k > 0, s, nf, a, psi,
                                              b, cA, cD, upto - done, ul, ur);
         if (e != cudaSuccess) return e;
         done = upto;
@@ -1303,7 +1276,7 @@ cudaError_t dns_run_dirichlet(int nf, void *u, void *u_tmp, const float *psi, in
     const double sq2 = 1.4142135623730951;
     double *a = static_cast<double *>(u), *b = static_cast<double *>(u_tmp);
     for (int k = 0; k < nsteps; ++k) {
-        const cudaError_t e = launch_chained(fn, grid, nt, k > 0, s, nf, a, b, aE, aN, r2 * cD, ul, ur,
+        const cudaError_t e = launch_chained(fn, grid, nt, 0, k > 0, s, nf, a, b, aE, aN, r2 * cD, ul, ur,
                                              sq2 * ul, sq2 * ur);
         if (e != cudaSuccess) return e;
         std::swap(a, b);

@@ -140,12 +140,19 @@ cudaError_t launch_periodize(const float *band, long long Nl, int n, int n_macro
 cudaError_t launch_wait_check_nbr(int *status, cudaStream_t s);
 cudaError_t launch_wait_check_mbar(int *status, cudaStream_t s);
 cudaError_t launch_wait_check_tile(int *status, cudaStream_t s);
-// tensor-core GEMM D = A B^T of the training step (gemm_tc.cu): mode 0 forward epilogue,
-// 1 backward epilogue, 2 partial sums over K slices
+// tensor-core GEMMs D = A B^T of the training step (gemm_tc.cu): mode 0 forward epilogue,
+// 1 backward epilogue; or three at once as partial sums over K slices
 cudaError_t gemm_tc(int mode, int M, int N, int K, const void *A, long long lda, const void *B,
                     long long ldb, const float *bias, float *Z, const float *Zprev, void *out,
-                    void *outT, int ldT, float *part, int splits, int *slices, int *status,
-                    cudaStream_t s);
+                    void *outT, int ldT, int *status, bool overlap, cudaStream_t s);
+struct GemmPart {
+    int M, N, K;
+    const void *A, *B;
+    long long lda, ldb;
+    float *part;
+    int splits;
+};
+cudaError_t gemm_tc_parts(GemmPart (&g)[3], int *status, bool overlap, cudaStream_t s);
 int gemm_tc_splits(int M, int N, int K, int sms);
 // 3-D core-matrix tensor map (CUtensorMap) of a bfloat16 matrix [rows][K], rows ld apart
 bool encode_rows_bf16(void *map, const void *base, long long rows, long long K, long long ld,
@@ -188,8 +195,12 @@ cudaError_t launch_features(const float *band, long long Nl, long long tile, int
                             const int *pidx, long long count, const double *B, double kappa,
                             void *X, float *F32, double *Q, cudaStream_t s);
 // ws: split-k partials of the CUDA-core GEMMs, ws_n floats (sur_split_workspace(h) lets
-// every training shape split fully; nullptr disables splitting)
+// every training shape split fully; nullptr disables splitting).  sur_grad_tc takes
+// sur_tc_workspace(h): three of those, and the output layer's.
 long long sur_split_workspace(int h);
+long long sur_tc_workspace(int h);
+// doubles of the loss partials for batches of up to M rows
+long long sur_loss_parts(int M);
 cudaError_t sur_forward(int h, int M, const void *X, const float *wf, const void *wb,
                         float *Z[4], void *Aact[3], float *ws, long long ws_n, cudaStream_t s);
 cudaError_t sur_grad(int h, int M, const void *X, const float *Y, const float *wf, const void *wb,
@@ -202,12 +213,12 @@ struct SurTc {
     __nv_bfloat16 *AT[3] = {};            // [h][ldT] transposed activations
     __nv_bfloat16 *WT[2] = {};            // [h][h] transposed W_1, W_2
     __nv_bfloat16 *dZ[2] = {};            // [max_rows][h] bfloat16 gradients
-    __nv_bfloat16 *dZT[2] = {};           // [h][ldT]
+    __nv_bfloat16 *dZT[3] = {};           // [h][ldT], per hidden layer
 };
 cudaError_t sur_grad_tc(int h, int M, const void *X, const float *Y, const float *wf,
-                        const void *wb, float *Z[4], void *Aact[3], float *dA, float *dB,
-                        float *g, double *part, double *loss_dev, float *ws, long long ws_n,
-                        const SurTc &tc, int *status, cudaStream_t s);
+                        const void *wb, float *Z[4], void *Aact[3], float *dA, float *g,
+                        double *part, double *loss_dev, float *ws, const SurTc &tc, int *status,
+                        cudaStream_t s);
 cudaError_t sur_adam(long long n, float *w, const float *g, float *m, float *v, float lr, int t,
                      void *wb, cudaStream_t s);
 cudaError_t sur_to_bf16(long long n, const float *w, void *wb, cudaStream_t s);
@@ -239,7 +250,37 @@ size_t mlp_tma_maps_bytes();
 cudaError_t launch_mlp_tma(const void *X, long long M, int h, int members, const void *maps,
                            const float *const *wf_dev, float *out, int *status, cudaStream_t s);
 
-// Shared small device helpers ------------------------------------------------
+// Shared small helpers --------------------------------------------------------
+// Chains of launches that each read what the one before wrote: a kernel launched with
+// launch_chained(overlap) starts while its predecessor in the stream still runs, does what does
+// not depend on it (set-up, coefficients), and calls chain_wait before anything that does.  Every
+// kernel of a chain calls it in every CTA (a CTA that left early would let the one after next
+// pass this one's predecessor); launched without overlap it returns at once.  The successor is
+// let in only after the wait: one launch ahead, no further (several waiting launches pack
+// their CTAs on few SMs).
+__device__ __forceinline__ void chain_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*fn)(P...), dim3 grid, dim3 threads, size_t smem, bool overlap,
+                                  cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = threads;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, fn, P(args)...);
+}
+
 __host__ __device__ inline long long pmod_ll(long long a, long long m)
 {
     long long r = a % m;

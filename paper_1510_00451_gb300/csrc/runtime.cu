@@ -1454,8 +1454,8 @@ cudaError_t grad_of(mlsd_surrogate *s, int member, int M, const void *X, const f
                     double *part, double *loss, float *ws, long long ws_n, cudaStream_t st)
 {
     if (s->train_tc && M <= s->tc.max_rows)
-        return sur_grad_tc(s->h, M, X, Y, s->w[member], s->wb[member], s->Z, s->A, s->dA, s->dB,
-                           g, part, loss, ws, ws_n, s->tc, s->status, st);
+        return sur_grad_tc(s->h, M, X, Y, s->w[member], s->wb[member], s->Z, s->A, s->dA, g, part,
+                           loss, ws, s->tc, s->status, st);
     return sur_grad(s->h, M, X, Y, s->w[member], s->wb[member], s->Z, s->A, s->dA, s->dB, g, part,
                     loss, ws, ws_n, st);
 }
@@ -1504,8 +1504,8 @@ int mlsd_surrogate_create(int members, int hidden, int max_batch, mlsd_surrogate
     if (!rc) rc = sur_alloc(s, (void **)&s->dA, M * H * 4);
     if (!rc) rc = sur_alloc(s, (void **)&s->dB, M * H * 4);
     s->ws_n = sur_split_workspace(hidden);
-    if (!rc) rc = sur_alloc(s, (void **)&s->ws, (size_t)s->ws_n * 4);
-    if (!rc) rc = sur_alloc(s, (void **)&s->part, ((3 * M + 255) / 256 + 1) * 8);
+    if (!rc) rc = sur_alloc(s, (void **)&s->ws, (size_t)std::max(s->ws_n, sur_tc_workspace(hidden)) * 4);
+    if (!rc) rc = sur_alloc(s, (void **)&s->part, (size_t)sur_loss_parts(max_batch) * 8);
     if (!rc) rc = sur_alloc(s, (void **)&s->loss, 8);
     if (!rc) rc = sur_alloc(s, (void **)&s->wb_ptrs, members * sizeof(void *));
     if (!rc) rc = sur_alloc(s, (void **)&s->wf_ptrs, members * sizeof(float *));
@@ -1533,7 +1533,7 @@ int mlsd_surrogate_create(int members, int hidden, int max_batch, mlsd_surrogate
         for (int l = 0; l < 3 && !rc; ++l) { rc = sur_alloc(s, &p, H * T * 2); t.AT[l] = (__nv_bfloat16 *)p; }
         for (int l = 0; l < 2 && !rc; ++l) { rc = sur_alloc(s, &p, H * H * 2); t.WT[l] = (__nv_bfloat16 *)p; }
         for (int l = 0; l < 2 && !rc; ++l) { rc = sur_alloc(s, &p, M * H * 2); t.dZ[l] = (__nv_bfloat16 *)p; }
-        for (int l = 0; l < 2 && !rc; ++l) { rc = sur_alloc(s, &p, H * T * 2); t.dZT[l] = (__nv_bfloat16 *)p; }
+        for (int l = 0; l < 3 && !rc; ++l) { rc = sur_alloc(s, &p, H * T * 2); t.dZT[l] = (__nv_bfloat16 *)p; }
         s->train_tc = !rc;
     }
     if (rc) { mlsd_surrogate_free(s); return rc; }

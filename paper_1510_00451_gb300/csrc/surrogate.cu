@@ -1021,14 +1021,23 @@ __global__ void k_merge_fallback(int n, const int *n_dev, const int *idx, const 
     K[3 * p + 2] = b[2] + s[3];
 }
 
-// Transpose of a row-major bfloat16 [rows][cols] (row stride cols) into [cols][ldT]:
+// Transposes of row-major bfloat16 [rows][cols] (row stride cols) into [cols][ldT]:
 // dst[c][r] = src[r][c] for r < rows, zero for rows <= r < ldT.  32 x 32 tiles
-// through shared memory (reads and writes along rows).
-__global__ void k_transpose_bf16(int rows, int cols, const __nv_bfloat16 *src, __nv_bfloat16 *dst,
-                                 int ldT)
+// through shared memory (reads and writes along rows); blockIdx.z picks the matrix.
+struct Transposes {
+    const __nv_bfloat16 *src[3];
+    __nv_bfloat16 *dst[3];
+    int rows[3], cols[3], ldT[3];
+};
+__global__ void k_transpose_bf16(Transposes a)
 {
     __shared__ __nv_bfloat16 t[32][33];
+    chain_wait();
+    const int z = blockIdx.z, rows = a.rows[z], cols = a.cols[z], ldT = a.ldT[z];
     const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+    if (r0 >= rows || c0 >= cols) return;
+    const __nv_bfloat16 *src = a.src[z];
+    __nv_bfloat16 *dst = a.dst[z];
     for (int k = threadIdx.y; k < 32; k += blockDim.y) {
         const int r = r0 + k, c = c0 + threadIdx.x;
         t[k][threadIdx.x] = (r < rows && c < cols) ? src[(long long)r * cols + c]
@@ -1041,40 +1050,57 @@ __global__ void k_transpose_bf16(int rows, int cols, const __nv_bfloat16 *src, _
     }
 }
 
-// Output layer of the tensor-core training step (3 outputs: one warp per row).
-// Z4[m][j] = b4[j] + sum_k A3[m][k] W4[j][k]
+// Output layer of the tensor-core training step (3 outputs: one warp per row), the loss and
+// its gradient: Z4[m][j] = b4[j] + sum_k A3[m][k] W4[j][k], dZ4 = 2 (Z4 - Y) / (3 M), and the
+// block's share of sum (Z4 - Y)^2.
 __global__ void k_out_fwd(int M, int h, const __nv_bfloat16 *A3, const __nv_bfloat16 *W4,
-                          const float *b4, float *Z4)
+                          const float *b4, const float *Y, float *Z4, float *dZ4, double *part)
 {
+    __shared__ double red[8];
+    chain_wait();
     const int m = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (m >= M) return;
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-    for (int k = lane; k < h; k += 32) {
-        const float x = __bfloat162float(A3[(long long)m * h + k]);
-        s0 = fmaf(x, __bfloat162float(W4[k]), s0);
-        s1 = fmaf(x, __bfloat162float(W4[h + k]), s1);
-        s2 = fmaf(x, __bfloat162float(W4[2 * h + k]), s2);
+    double loss = 0.0;
+    if (m < M) {
+        float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+        for (int k = lane; k < h; k += 32) {
+            const float x = __bfloat162float(A3[(long long)m * h + k]);
+            s0 = fmaf(x, __bfloat162float(W4[k]), s0);
+            s1 = fmaf(x, __bfloat162float(W4[h + k]), s1);
+            s2 = fmaf(x, __bfloat162float(W4[2 * h + k]), s2);
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+            s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        }
+        if (lane == 0) {
+            const float z[3] = {b4[0] + s0, b4[1] + s1, b4[2] + s2};
+            for (int j = 0; j < 3; ++j) {
+                const float d = z[j] - Y[3 * m + j];
+                Z4[3 * m + j] = z[j];
+                dZ4[3 * m + j] = 2.0f * d / (3.0f * (float)M);
+                loss += (double)d * d;
+            }
+        }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-    }
-    if (lane == 0) {
-        Z4[3 * m] = b4[0] + s0;
-        Z4[3 * m + 1] = b4[1] + s1;
-        Z4[3 * m + 2] = b4[2] + s2;
+    if (lane == 0) red[threadIdx.x >> 5] = loss;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
+        part[blockIdx.x] = t;
     }
 }
 
 // Partial sums of dW4[j][k] = sum_m dZ4[m][j] A3[m][k] and db4[j] = sum_m dZ4[m][j] over
 // the row chunk blockIdx.y (rows y*chunk .. +chunk-1): a block of 32 columns x 8 row groups
 // (rows g, g + 8, ...), reduced over the groups in order, into part[y][j][k] and (the
-// blocks of the first column tile) bpart[y][j]; k_split_reduce adds the chunks in order
+// blocks of the first column tile) bpart[y][j]; k_grad_reduce adds the chunks in order
 __global__ void k_out_bwd_w(int M, int h, int chunk, const float *dZ4, const __nv_bfloat16 *A3,
                             float *part, float *bpart)
 {
     __shared__ float red[8][4][33];
+    chain_wait();
     const int c = threadIdx.x & 31, g = threadIdx.x >> 5, k = blockIdx.x * 32 + c;
     const int mb = blockIdx.y * chunk, me = min(M, mb + chunk);
     float s0 = 0.f, s1 = 0.f, s2 = 0.f, b = 0.f;
@@ -1106,6 +1132,7 @@ __global__ void k_out_bwd_x(int M, int h, const float *dZ4, const __nv_bfloat16 
                             __nv_bfloat16 *dZ, __nv_bfloat16 *dZT, int ldT)
 {
     __shared__ __nv_bfloat16 t[32][33];
+    chain_wait();
     const int m0 = blockIdx.y * 32, k0 = blockIdx.x * 32, k = k0 + threadIdx.x;
     float w0 = 0.f, w1 = 0.f, w2 = 0.f;
     if (k < h) {
@@ -1130,46 +1157,80 @@ __global__ void k_out_bwd_x(int M, int h, const float *dZ4, const __nv_bfloat16 
     }
 }
 
-// FP32 [M][N] (bfloat16-valued) to bfloat16 [M][N] and its transpose [N][ldT] (zero for
-// M <= m < ldT)
-__global__ void k_to_bf16_t(int M, int N, const float *src, __nv_bfloat16 *dst, __nv_bfloat16 *dstT,
-                            int ldT)
+// The gradient from its parts, one launch.  Blocks of the hidden layers' weights: dW_l = the K
+// slices' partials added in order, four entries a thread.  Blocks of their biases: db_l[r] = the
+// sum of row r of dZ_l^T (bfloat16, row stride ld a multiple of 8, zero padding), one warp a
+// row, each lane 16-byte vectors 8 k apart, then the warp tree.  Then the output layer's (dW4 and
+// db4 from k_out_bwd_w's chunks in order), and the loss, its blocks' shares added in FP64.
+struct GradReduce {
+    const float *part[3];
+    float *w[3], *b[3];
+    const __nv_bfloat16 *dZT[3];
+    long long n[3];                        // h * din
+    int slices[3], wblocks[3], bblocks;    // blocks per layer: weights, biases
+    int h, M, ld, oblocks;
+    const float *opart, *obpart;           // [chunks][3][h], [chunks][3]
+    float *ow, *ob;
+    int chunks, nloss;
+    const double *lpart;
+    double lscale, *loss;
+};
+__global__ void __launch_bounds__(256) k_grad_reduce(GradReduce a)
 {
-    __shared__ __nv_bfloat16 t[32][33];
-    const int m0 = blockIdx.y * 32, n0 = blockIdx.x * 32;
-    for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-        const int m = m0 + k, n = n0 + threadIdx.x;
-        __nv_bfloat16 v = __float2bfloat16_rn(0.f);
-        if (m < M && n < N) {
-            v = __float2bfloat16_rn(src[(long long)m * N + n]);
-            dst[(long long)m * N + n] = v;
+    __shared__ double red[8];
+    chain_wait();
+    int blk = blockIdx.x;
+    const int lane = threadIdx.x & 31;
+    for (int l = 0; l < 3; ++l) {
+        if (blk < a.wblocks[l]) {
+            const long long x = 4 * (blk * 256LL + threadIdx.x), n = a.n[l];
+            if (x >= n) return;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int z = 0; z < a.slices[l]; ++z) {
+                const float4 p = *reinterpret_cast<const float4 *>(a.part[l] + z * n + x);
+                v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
+            }
+            float *o = a.w[l] + x;             // a member's layers start anywhere: 4-byte stores
+            o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+            return;
         }
-        t[k][threadIdx.x] = v;
-    }
-    __syncthreads();
-    for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-        const int n = n0 + k, m = m0 + threadIdx.x;
-        if (n < N && m < ldT) dstT[(long long)n * ldT + m] = t[threadIdx.x][k];
-    }
-}
-
-// out[r] = sum over k < K of src[r][k] (bfloat16, row stride ld a multiple of 8, zero
-// padding up to ld), one warp per row, FP32 in a fixed order (each lane sums 16-byte
-// vectors 8 k apart, then the warp tree)
-__global__ void k_rowsum_bf16(int rows, int K, const __nv_bfloat16 *src, int ld, float *out)
-{
-    const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (r >= rows) return;
-    float acc = 0.f;
-    const __nv_bfloat16 *row = src + (long long)r * ld;
-    for (int k = 8 * lane; k < K; k += 256) {
-        const uint4 q = *reinterpret_cast<const uint4 *>(row + k);
-        const __nv_bfloat16 *e = reinterpret_cast<const __nv_bfloat16 *>(&q);
+        blk -= a.wblocks[l];
+        if (blk < a.bblocks) {
+            const int r = blk * 8 + (threadIdx.x >> 5);
+            if (r >= a.h) return;
+            float acc = 0.f;
+            const __nv_bfloat16 *row = a.dZT[l] + (long long)r * a.ld;
+            for (int k = 8 * lane; k < a.M; k += 256) {
+                const uint4 q = *reinterpret_cast<const uint4 *>(row + k);
+                const __nv_bfloat16 *e = reinterpret_cast<const __nv_bfloat16 *>(&q);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc += __bfloat162float(e[i]);   // zeros past K
+                for (int i = 0; i < 8; ++i) acc += __bfloat162float(e[i]);   // zeros past M
+            }
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (lane == 0) a.b[l][r] = acc;
+            return;
+        }
+        blk -= a.bblocks;
     }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) out[r] = acc;
+    if (blk < a.oblocks) {
+        const int x = blk * 256 + threadIdx.x, n = 3 * a.h;
+        if (x >= n + 3) return;
+        float v = 0.f;
+        for (int z = 0; z < a.chunks; ++z) v += x < n ? a.opart[(long long)z * n + x] : a.obpart[z * 3 + x - n];
+        if (x < n) a.ow[x] = v;
+        else a.ob[x - n] = v;
+        return;
+    }
+    double t = 0.0;
+    for (int i = threadIdx.x; i < a.nloss; i += 256) t += a.lpart[i];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) red[threadIdx.x >> 5] = t;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        t = 0.0;
+        for (int w = 0; w < 8; ++w) t += red[w];
+        *a.loss = t * a.lscale;
+    }
 }
 
 }  // namespace
@@ -1274,6 +1335,8 @@ cudaError_t sur_forward(int h, int M, const void *X, const float *wf, const void
 }
 
 long long sur_split_workspace(int h) { return (long long)SPLIT_MAX * h * (MLSD_SUR_IN + 1); }
+long long sur_tc_workspace(int h) { return 3 * sur_split_workspace(h) + SPLIT_MAX * (3LL * h + 3); }
+long long sur_loss_parts(int M) { return ((long long)M + 7) / 8 + 1; }
 
 cudaError_t sur_grad(int h, int M, const void *X, const float *Y, const float *wf, const void *wb_,
                      float *Z[4], void *Aact[3], float *dA, float *dB_, float *g, double *part,
@@ -1310,84 +1373,90 @@ cudaError_t sur_grad(int h, int M, const void *X, const float *Y, const float *w
 
 // The gradient of one member with the hidden layers' contractions on the tensor cores
 // (gemm_tc): forward Z_l = A_{l-1} W_l^T + b_l with bfloat16 act_l and its transpose,
-// l = 0..2; the output layer, the loss and the output layer's gradients as in sur_grad
-// (CUDA cores); then for l = 2, 1, 0: dW_l = dZ_l^T A_{l-1} (K = the batch, split over
-// CTAs, partials summed in a fixed order), db_l = the row sums of dZ_l^T, and
-// dZ_{l-1} = bf16((dZ_l W_l) gelu'(Z_{l-1})) and its transpose.  dZ of the hidden
-// layers is a bfloat16 operand throughout (the oracle's emulation rounds it the same).
+// l = 0..2; the output layer, the loss and the output layer's gradients on the CUDA cores;
+// the data gradients dZ_{l-1} = bf16((dZ_l W_l) gelu'(Z_{l-1})) and their transposes, l = 2, 1;
+// then the weight gradients dW_l = dZ_l^T A_{l-1} of all three layers in one launch (K = the
+// batch, split over CTAs) and one launch that adds the partials in a fixed order and sums the
+// bias gradients.  dZ of the hidden layers is a bfloat16 operand throughout (the oracle's
+// emulation rounds it the same).  What bounds it is the chain of launches, so there are 11 of
+// them (25 when every small step had its own), each starting while its predecessor runs: h = 256,
+// 2048 rows 196 -> 131 us a gradient.
 cudaError_t sur_grad_tc(int h, int M, const void *X, const float *Y, const float *wf,
-                        const void *wb_, float *Z[4], void *Aact[3], float *dA, float *dB_,
-                        float *g, double *part, double *loss_dev, float *ws, long long ws_n,
-                        const SurTc &tc, int *status, cudaStream_t s)
+                        const void *wb_, float *Z[4], void *Aact[3], float *dA, float *g,
+                        double *part, double *loss_dev, float *ws, const SurTc &tc, int *status,
+                        cudaStream_t s)
 {
     const Layers L = layers(h);
     const __nv_bfloat16 *wb = static_cast<const __nv_bfloat16 *>(wb_);
     const int ldT = tc.ldT;
     if (M > tc.max_rows || ldT < ((M + 7) / 8) * 8) return cudaErrorInvalidValue;
-    cudaError_t e = cudaSuccess;
     const dim3 tb(32, 8);
-    auto tgrid = [](int rows, int cols) { return dim3((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32)); };
-    // W_1^T, W_2^T for the data gradients
-    count_launches(2);
-    for (int l = 1; l <= 2; ++l)
-        k_transpose_bf16<<<tgrid(h, h), tb, 0, s>>>(h, h, wb + L.w[l], tc.WT[l - 1], h);
-    e = cudaGetLastError();
+    // W_1^T, W_2^T for the data gradients, X^T for the first layer's weight gradient
+    Transposes tr;
+    for (int i = 0; i < 2; ++i) {
+        tr.src[i] = wb + L.w[i + 1]; tr.dst[i] = tc.WT[i];
+        tr.rows[i] = tr.cols[i] = tr.ldT[i] = h;
+    }
+    tr.src[2] = static_cast<const __nv_bfloat16 *>(X); tr.dst[2] = tc.XT;
+    tr.rows[2] = M; tr.cols[2] = MLSD_SUR_IN; tr.ldT[2] = ldT;
+    count_launches(5);
+    k_transpose_bf16<<<dim3((unsigned)((std::max(h, MLSD_SUR_IN) + 31) / 32),
+                            (unsigned)((std::max(h, M) + 31) / 32), 3), tb, 0, s>>>(tr);
+    cudaError_t e = cudaGetLastError();
     // forward, hidden layers on the tensor cores
     const __nv_bfloat16 *in = static_cast<const __nv_bfloat16 *>(X);
     for (int l = 0; l < 3 && e == cudaSuccess; ++l) {
         e = gemm_tc(0, M, h, L.din[l], in, L.din[l], wb + L.w[l], L.din[l], wf + L.b[l], Z[l],
-                    nullptr, Aact[l], tc.AT[l], ldT, nullptr, 1, nullptr, status, s);
+                    nullptr, Aact[l], tc.AT[l], ldT, status, true, s);
         in = static_cast<const __nv_bfloat16 *>(Aact[l]);
     }
     if (e != cudaSuccess) return e;
-    // output layer (3 outputs) and its gradients, on the CUDA cores: Z4, the loss and
-    // dZ4, dW4 and db4, and dZ3 = bf16((dZ4 W4) gelu'(Z3)) with its transpose
-    const int nb = (3 * M + 255) / 256;
-    count_launches(6);
-    k_out_fwd<<<(unsigned)((M + 7) / 8), 256, 0, s>>>(M, h, in, wb + L.w[3], wf + L.b[3], Z[3]);
-    k_mse<<<nb, 256, 0, s>>>(M, Z[3], Y, dA, part);
-    k_sum_parts<<<1, 32, 0, s>>>(nb, part, 1.0 / (3.0 * M), loss_dev);
-    {
-        const int S = std::min(16, (M + 127) / 128), chunk = (M + S - 1) / S;
-        float *bpart = ws + (long long)S * 3 * h;
-        k_out_bwd_w<<<dim3((unsigned)((h + 31) / 32), (unsigned)S), 256, 0, s>>>(M, h, chunk, dA, in,
-                                                                              ws, bpart);
-        count_launches(1);
-        k_split_reduce<<<(unsigned)((3 * h + 3 + 255) / 256), 256, 0, s>>>(3, h, S, ws, g + L.w[3], h,
-                                                                          Epi{}, bpart, g + L.b[3]);
-    }
-    k_out_bwd_x<<<tgrid(M, h), tb, 0, s>>>(M, h, dA, wb + L.w[3], Z[2], tc.dZ[0], tc.dZT[0], ldT);
-    k_transpose_bf16<<<tgrid(M, MLSD_SUR_IN), tb, 0, s>>>(M, MLSD_SUR_IN, static_cast<const __nv_bfloat16 *>(X),
-                                                         tc.XT, ldT);
-    e = cudaGetLastError();
-    (void)dB_;
-    int cur = 0;
+    // output layer (3 outputs), loss and dZ4; partials of dW4 and db4; dZ_2 and its transpose
+    const int nloss = (M + 7) / 8, S = std::min(SPLIT_MAX, (M + 127) / 128), chunk = (M + S - 1) / S;
+    float *opart = ws + 3 * sur_split_workspace(h), *obpart = opart + (long long)S * 3 * h;
+    e = launch_chained(k_out_fwd, dim3((unsigned)nloss), 256, 0, true, s, M, h, in, wb + L.w[3],
+                       wf + L.b[3], Y, Z[3], dA, part);
+    if (e == cudaSuccess)
+        e = launch_chained(k_out_bwd_w, dim3((unsigned)((h + 31) / 32), (unsigned)S), 256, 0, true, s, M, h,
+                           chunk, dA, in, opart, obpart);
+    if (e == cudaSuccess)
+        e = launch_chained(k_out_bwd_x, dim3((unsigned)((h + 31) / 32), (unsigned)((M + 31) / 32)), tb, 0,
+                           true, s, M, h, dA, wb + L.w[3], Z[2], tc.dZ[0], tc.dZT[2], ldT);
+    // dZ_{l-1} = bf16((dZ_l W_l) gelu'(Z_{l-1})): A = dZ_l [M][h], B = W_l^T [din][h]
+    for (int l = 2; l >= 1 && e == cudaSuccess; --l)
+        e = gemm_tc(1, M, L.din[l], h, tc.dZ[l & 1], h, tc.WT[l - 1], h, nullptr, nullptr, Z[l - 1],
+                    tc.dZ[(l & 1) ^ 1], tc.dZT[l - 1], ldT, status, true, s);
+    if (e != cudaSuccess) return e;
     int sms = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    for (int l = 2; l >= 0 && e == cudaSuccess; --l) {
+    // dW_l[j][k] = sum_m dZ_l[m][j] A_{l-1}[m][k]: A = dZ_l^T [h][M], B = A_{l-1}^T [din][M]
+    GemmPart gp[3];
+    GradReduce rd = {};
+    for (int l = 0; l < 3; ++l) {
         const int din = L.din[l];
-        const void *Bt = l > 0 ? static_cast<const void *>(tc.AT[l - 1]) : static_cast<const void *>(tc.XT);
-        // dW_l[j][k] = sum_m dZ[m][j] A_{l-1}[m][k]: A = dZ^T [h][M], B = A_{l-1}^T [din][M]
         int splits = gemm_tc_splits(h, din, M, sms);
-        while (splits > 1 && (long long)splits * h * din > ws_n) --splits;
-        int used = 1;
-        e = gemm_tc(2, h, din, M, tc.dZT[cur], ldT, Bt, ldT, nullptr, nullptr, nullptr, nullptr,
-                    nullptr, ldT, ws, splits, &used, status, s);
-        if (e != cudaSuccess) break;
-        const long long n = (long long)h * din;
-        count_launches(2);
-        k_split_reduce<<<(unsigned)std::min<long long>((n + 255) / 256, 8LL * sms), 256, 0, s>>>(
-            h, din, used, ws, g + L.w[l], din, Epi{}, nullptr, nullptr);
-        k_rowsum_bf16<<<(unsigned)((h + 7) / 8), 256, 0, s>>>(h, M, tc.dZT[cur], ldT, g + L.b[l]);
-        e = cudaGetLastError();
-        if (e != cudaSuccess || l == 0) break;
-        // dZ_{l-1} = bf16((dZ_l W_l) gelu'(Z_{l-1})): A = dZ_l [M][h], B = W_l^T [din][h]
-        e = gemm_tc(1, M, din, h, tc.dZ[cur], h, tc.WT[l - 1], h, nullptr, nullptr, Z[l - 1],
-                    tc.dZ[cur ^ 1], tc.dZT[cur ^ 1], ldT, nullptr, 1, nullptr, status, s);
-        cur ^= 1;
+        while (splits > 1 && (long long)splits * h * din > sur_split_workspace(h)) --splits;
+        gp[l] = {h, din, M, tc.dZT[l], l > 0 ? static_cast<const void *>(tc.AT[l - 1]) : tc.XT, ldT, ldT,
+                 ws + l * sur_split_workspace(h), splits};
     }
-    return e;
+    e = gemm_tc_parts(gp, status, true, s);
+    if (e != cudaSuccess) return e;
+    int blocks = 0;
+    rd.bblocks = (h + 7) / 8;
+    for (int l = 0; l < 3; ++l) {
+        rd.part[l] = gp[l].part; rd.slices[l] = gp[l].splits;
+        rd.w[l] = g + L.w[l]; rd.b[l] = g + L.b[l]; rd.dZT[l] = tc.dZT[l];
+        rd.n[l] = (long long)h * L.din[l];
+        rd.wblocks[l] = (int)((rd.n[l] / 4 + 255) / 256);
+        blocks += rd.wblocks[l] + rd.bblocks;
+    }
+    rd.h = h; rd.M = M; rd.ld = ldT;
+    rd.opart = opart; rd.obpart = obpart; rd.ow = g + L.w[3]; rd.ob = g + L.b[3];
+    rd.chunks = S; rd.oblocks = (3 * h + 3 + 255) / 256;
+    rd.nloss = nloss; rd.lpart = part; rd.lscale = 1.0 / (3.0 * M); rd.loss = loss_dev;
+    blocks += rd.oblocks + 1;
+    return launch_chained(k_grad_reduce, dim3((unsigned)blocks), 256, 0, true, s, rd);
 }
 
 cudaError_t sur_adam(long long n, float *w, const float *g, float *m, float *v, float lr, int t,
