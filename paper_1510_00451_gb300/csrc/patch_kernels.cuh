@@ -1032,8 +1032,8 @@ struct Tile {
         }
         const long long Nl = prm.Nl;
         const long long pi = p % prm.n_macro, pj = p / prm.n_macro;
-        const long long ox = patch_origin(pi, prm.n_macro, Nl, N);
-        const long long oy = patch_origin(pj, prm.n_macro, Nl, N);
+        const long long ox = pmod_ll(patch_origin(pi, prm.n_macro, Nl, N), Nl);
+        const long long oy = pmod_ll(patch_origin(pj, prm.n_macro, Nl, N), Nl);
 
         // ---- set-up: psi rows g0-1 .. g0+NS (patch-periodic), velocity, time step --
         real *psi = sm;
@@ -1553,8 +1553,8 @@ struct Tile64 {
         const int a0 = tx * BX, b0 = ty * BY;
         double *red = sm + RED, *arr = sm + ARR;
         const long long Nl = prm.Nl;
-        const long long ox = patch_origin(p % prm.n_macro, prm.n_macro, Nl, N);
-        const long long oy = patch_origin(p / prm.n_macro, prm.n_macro, Nl, N);
+        const long long ox = pmod_ll(patch_origin(p % prm.n_macro, prm.n_macro, Nl, N), Nl);
+        const long long oy = pmod_ll(patch_origin(p / prm.n_macro, prm.n_macro, Nl, N), Nl);
         // ---- set-up as Tile::run: psi, velocity, time step ----
         double *psi = sm;
         const double *band = static_cast<const double *>(prm.band);
@@ -1822,8 +1822,8 @@ struct Tile2 {
         const int a0 = tx * BX, b0 = ty * BY;
         double *red = reinterpret_cast<double *>(sm + S::WORDS);
         const long long Nl = prm.Nl;
-        const long long ox = patch_origin(p % prm.n_macro, prm.n_macro, Nl, N);
-        const long long oy = patch_origin(p / prm.n_macro, prm.n_macro, Nl, N);
+        const long long ox = pmod_ll(patch_origin(p % prm.n_macro, prm.n_macro, Nl, N), Nl);
+        const long long oy = pmod_ll(patch_origin(p / prm.n_macro, prm.n_macro, Nl, N), Nl);
         float *psi = reinterpret_cast<float *>(sm);
         const float *band = static_cast<const float *>(prm.band);
         for (int c = tid; c < N * N; c += NT) {
