@@ -888,22 +888,95 @@ __global__ void k_dns_vmax(int nf, const float *psi, float ax, unsigned *out)
     if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(m));
 }
 
-// box average onto the macro grid; box[j*N+i] = FP64 sum of the box
-__global__ void k_coarse(int nf, const float *u, int N, float *U, double *box)
+// Box average onto the macro grid; box[j*N+i] = FP64 sum of the box.  W warps a box, PER nodes a
+// lane at a time, each read once.  An SM issues 2 FP64 operations a clock: converting and adding
+// every node in FP64 took 8 times as long as reading it.  So up to T PER nodes at a time are
+// added as integers: with E the largest exponent of the n <= 2^bits nodes and shift = 38 - bits,
+// each becomes its 24-bit significand in units of 2^(E - 150 - shift), so that n of them fit
+// 62 bits.  Nodes within 2^shift (2^26 at least) of the largest are added exactly, smaller ones
+// rounded to the unit (2^-49 of the largest at most), and the sum is rounded once to FP64.
+// Infinities and NaN are added in FP64.  The 8 warps' FP64 work is left to one of them (a warp
+// with one box takes as long as one with 8).  8192^2 onto 64^2, 128^2, 512^2: 288, 367, 2081 us
+// for a CTA a box in FP64, 118, 122, 144 so (reading them once: 40).  What bounds it: the integer
+// operations, about 25 a node.
+template <int W, int PER>
+__global__ void __launch_bounds__(256) k_coarse(int nf, const float *__restrict__ u, int N, float *U,
+                                                double *box, int bits)
 {
-    __shared__ double red[32];
-    const int i = blockIdx.x, j = blockIdx.y, r = nf / N;
-    double s = 0.0;
-    for (int k = threadIdx.x; k < r * r; k += blockDim.x) {
-        const int db = k / r, da = k % r;
-        int b = j * r - r / 2 + db; b = b < 0 ? b + nf : (b >= nf ? b - nf : b);
-        int a = i * r - r / 2 + da; a = a < 0 ? a + nf : (a >= nf ? a - nf : a);
-        s += (double)u[(long long)b * nf + a];
+    constexpr int T = 32 * W, BOXES = 8 / W;          // threads per box, boxes per CTA
+    __shared__ unsigned tops[8];
+    __shared__ long long accs[8];
+    __shared__ double sums[8];
+    const int r = nf / N, n = r * r, t = threadIdx.x % T, warp = threadIdx.x >> 5, w0 = warp / W * W;
+    const long long b = (long long)blockIdx.x * BOXES + threadIdx.x / T;
+    const bool in = b < (long long)N * N;
+    const int i = (int)(b % N), j = (int)(b / N), x0 = i * r - r / 2, y0 = j * r - r / 2;
+    const int sx = T % r, sy = T / r, shift = 38 - bits;
+    // thread k < BOXES: the sum of the CTA's k-th box.  One chunk of nodes unless W = 8
+    double total = 0.0;
+    int x = t % r, y = t / r;
+    for (int base = 0; base < (W < 8 ? 1 : n); base += T * PER) {
+        // the lane's nodes: every T-th of the box's, row by row
+        unsigned v[PER], top = 0;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            int gx = x0 + x, gy = y0 + y;
+            gx = gx < 0 ? gx + nf : gx;                // a box reaches past the grid's start only
+            gy = gy < 0 ? gy + nf : gy;
+            v[k] = in && base + t + k * T < n ? __float_as_uint(__ldg(u + (long long)gy * nf + gx)) : 0u;
+            x += sx;
+            y += sy;
+            if (x >= r) { x -= r; ++y; }
+        }
+#pragma unroll
+        for (int k = 0; k < PER; ++k) top = max(top, v[k] & 0x7fffffffu);
+        top = __reduce_max_sync(0xffffffffu, top);
+        if ((threadIdx.x & 31) == 0) tops[warp] = top;
+        if constexpr (W > 1) {
+            __syncthreads();
+#pragma unroll
+            for (int w = 0; w < W; ++w) top = max(top, tops[w0 + w]);
+        }
+        const int E = max(1, (int)(top >> 23));        // denormals: the exponent of 2^-126
+        long long acc = 0;
+        if (E < 255) {
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                const int e = (v[k] >> 23) & 255, sh = shift - (E - max(1, e));
+                const unsigned long long m = (v[k] & 0x7fffffu) | (e ? 0x800000u : 0u);
+                long long q = 0;
+                if (sh >= 0) q = (long long)(m << sh);
+                else if (sh > -25) q = (long long)((m + (1ull << (-sh - 1))) >> -sh);
+                acc += (v[k] >> 31) ? -q : q;
+            }
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if ((threadIdx.x & 31) == 0) accs[warp] = acc;
+        } else {
+            double s = 0.0;
+#pragma unroll
+            for (int k = 0; k < PER; ++k) s += (double)__uint_as_float(v[k]);
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if ((threadIdx.x & 31) == 0) sums[warp] = s;
+        }
+        __syncthreads();
+        if (threadIdx.x < BOXES) {
+            unsigned tb = 0;
+            long long a = 0;
+            for (int w = 0; w < W; ++w) tb = max(tb, tops[threadIdx.x * W + w]);
+            const int Eb = max(1, (int)(tb >> 23));
+            if (Eb < 255) {
+                for (int w = 0; w < W; ++w) a += accs[threadIdx.x * W + w];
+                total += ldexp((double)a, Eb - 150 - shift);
+            } else {
+                for (int w = 0; w < W; ++w) total += sums[threadIdx.x * W + w];
+            }
+        }
+        if constexpr (W == 8) __syncthreads();
     }
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) {
-        U[j * N + i] = (float)(s / ((double)r * r));
-        if (box) box[j * N + i] = s;
+    const long long bo = (long long)blockIdx.x * BOXES + threadIdx.x;
+    if (threadIdx.x < BOXES && bo < (long long)N * N) {
+        U[bo] = (float)(total / ((double)r * r));
+        if (box) box[bo] = total;
     }
 }
 
@@ -1304,7 +1377,13 @@ cudaError_t coarse_grain(int nf, const float *u, int N, float *U, double *mass_d
 {
     double *box = mass_dev ? mass_dev + 1 : nullptr;
     count_launches(mass_dev ? 2 : 1);
-    k_coarse<<<dim3(N, N), 256, 0, s>>>(nf, u, N, U, box);
+    const int r = nf / N;
+    int bits = 0;                                      // of a chunk's nodes: 4096 at most
+    while (bits < 12 && (1 << bits) < r * r) ++bits;
+    const long long boxes = (long long)N * N;
+    if (r <= 16) k_coarse<1, 8><<<(unsigned)((boxes + 7) / 8), 256, 0, s>>>(nf, u, N, U, box, bits);
+    else if (r <= 32) k_coarse<2, 16><<<(unsigned)((boxes + 3) / 4), 256, 0, s>>>(nf, u, N, U, box, bits);
+    else k_coarse<8, 16><<<(unsigned)boxes, 256, 0, s>>>(nf, u, N, U, box, bits);
     if (mass_dev) {
         const double h = 2.0 * kPi / nf;
         k_sum<<<1, 1024, 0, s>>>(N * N, box, h * h, mass_dev);

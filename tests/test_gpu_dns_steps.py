@@ -65,3 +65,41 @@ def test_grid_psi_edges(mlsd, torch_mod, nf):
     mlsd.grid_psi(spec, nf, g)
     ref = oracle.grid_psi(spec, nf)
     assert np.abs(g.cpu().numpy() - ref).max() < 1e-6 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("r,N", [(1, 5), (2, 3), (3, 4), (7, 9), (31, 2), (33, 3), (64, 3), (65, 2), (100, 1)])
+@pytest.mark.parametrize("kind", ["normal", "cancelling", "wide", "denormal"])
+def test_box_averages(mlsd, torch_mod, r, N, kind):
+    # U against the exact sum of each box: one rounding to FP32, and the sum's own error, at most
+    # half a unit of 2^-48 of the largest node per node (fixed point) or 2^-53 n of it (FP64)
+    rng = np.random.default_rng(r)
+    nf = r * N
+    u = rng.standard_normal((nf, nf))
+    if kind == "cancelling":
+        u = 1e6 * (u - u.mean()) + 1.0
+    if kind == "wide":
+        u *= 10.0 ** rng.uniform(-30, 5, u.shape)
+    if kind == "denormal":
+        u *= 1e-40
+    u = u.astype(np.float32)
+    U = torch_mod.full((N, N), 7.0, dtype=torch_mod.float32, device="cuda:0")
+    m = mlsd.coarse_grain(torch_mod.tensor(u, device="cuda:0"), N, U)
+    ul = np.roll(u.astype(np.longdouble), (r // 2, r // 2), (0, 1)).reshape(N, r, N, r)
+    box, top = ul.sum((1, 3)), np.abs(ul).max((1, 3))
+    ref = box / (r * r)
+    tol = np.abs(ref) * 2.0**-24 * 1.01 + top * 2.0**-38 * 2.0**-10 + 2.0**-150
+    assert np.all(np.abs(U.cpu().numpy() - ref) <= tol)
+    h = 2 * np.pi / nf
+    assert abs(m - box.sum() * h * h) <= h * h * nf * nf * float(top.max()) * 2.0**-46
+
+
+@pytest.mark.parametrize("r", [4, 65])
+def test_box_averages_not_finite(mlsd, torch_mod, r):
+    # boxes reach half a side back: node (0, 0) and node (r, 2 r) are inside boxes (0, 0) and (1, 2)
+    u = torch_mod.ones(3 * r, 3 * r, dtype=torch_mod.float32, device="cuda:0")
+    u[0, 0], u[r, 2 * r], u[r, 0], u[r, 1] = float("nan"), float("-inf"), float("inf"), float("-inf")
+    U = torch_mod.empty(3, 3, dtype=torch_mod.float32, device="cuda:0")
+    mlsd.coarse_grain(u, 3, U, want_mass=False)
+    V = U.cpu().numpy()
+    assert np.isnan(V[0, 0]) and V[1, 2] == -np.inf and np.isnan(V[1, 0])
+    assert np.all(V[[0, 0, 1, 2, 2, 2], [1, 2, 1, 0, 1, 2]] == 1.0)
