@@ -52,4 +52,15 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void *map, int x
         :: "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(mbar) : "memory");
 }
 
+// Matrix descriptor of a K-major bfloat16 operand tile that a 2-D copy with the 128-byte swizzle
+// staged: rows of 64 elements (128 bytes), 8 rows a swizzle atom of 1024 bytes, atoms one after
+// the other.  addr: the tile (1024-byte aligned) plus 32 bytes per 16 elements along K.
+// Boxes of 128-byte rows arrive several times faster than core-matrix boxes of 16-byte rows, which
+// paced every GEMM here.
+__device__ __forceinline__ uint64_t desc_sw128(uint32_t addr)
+{
+    return (uint64_t)((addr >> 4) & 0x3FFFu) | (uint64_t)1 << 16 | (uint64_t)(1024 >> 4) << 32 |
+           (uint64_t)1 << 46 | (uint64_t)2 << 61;
+}
+
 }  // namespace mlsd

@@ -2,7 +2,7 @@
 //   D[M][N] = A[M][K] B[N][K]^T, A and B bfloat16 with K contiguous (K-major),
 //   FP32 accumulation in tensor memory, one 128 x BN output tile per CTA and
 //   optionally one slice of K per CTA (gridDim.z slices, partial sums).
-// Operands arrive by cp.async.bulk.tensor through 3-D core-matrix views into a
+// Operands arrive by cp.async.bulk.tensor with the 128-byte swizzle into a
 // ring of mbarrier-guarded slots (6 of 32 KB, or 4 of 48 KB for 256-column tiles); one thread issues the MMAs
 // (kind::f16, M = 128, N = BN, K = 16 per instruction) and commits each slot's
 // release and the accumulator; the epilogue reads the accumulator rows with
@@ -22,6 +22,7 @@
 #include <cstdint>
 #include <cstdlib>
 
+#include "async_copy.cuh"
 #include "mlsd_internal.cuh"
 
 namespace mlsd {
@@ -57,17 +58,6 @@ __device__ __forceinline__ uint32_t s_u32(const void *p)
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// no-swizzle K-major shared-memory matrix descriptor (tcgen05 version bit set)
-__device__ __forceinline__ uint64_t gt_desc(uint32_t addr, uint32_t lbo, uint32_t sbo)
-{
-    uint64_t d = 0;
-    d |= (uint64_t)((addr >> 4) & 0x3FFFu);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-    d |= (uint64_t)1 << 46;
-    return d;
-}
-
 // instruction descriptor: D FP32, A and B bfloat16, both K-major, M x N
 __device__ __forceinline__ uint32_t gt_idesc(int M, int N)
 {
@@ -88,16 +78,6 @@ __device__ __forceinline__ bool gt_wait(uint32_t mbar, uint32_t parity)
         if (ok) return true;
         if (clock64() - t0 > kGtWaitClocks) return false;
     }
-}
-
-__device__ __forceinline__ void gt_tma3(uint32_t dst, const CUtensorMap *map, int c1, int c2,
-                                        uint32_t mbar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4}], [%5];"
-        :: "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(c1), "r"(c2), "r"(mbar)
-        : "memory");
 }
 
 __device__ __forceinline__ float gt_gelu(float z)
@@ -123,7 +103,8 @@ __global__ void __launch_bounds__(GT_THREADS, 1) k_gemm_tc(const __grid_constant
     constexpr int A_BYTES = GT_M * GT_KC * 2, B_BYTES = BN * GT_KC * 2, SLOT = A_BYTES + B_BYTES;
     constexpr int GT_RING = gt_ring<BN>();
     constexpr uint32_t TCOLS = BN <= 32 ? 32 : (BN <= 64 ? 64 : (BN <= 128 ? 128 : 256));
-    extern __shared__ __align__(1024) unsigned char smem[];
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char *smem = smem_raw + ((1024 - (s_u32(smem_raw) & 1023)) & 1023);   // swizzle atoms
     __shared__ __align__(8) uint64_t full[GT_RING], empty[GT_RING], accb;
     __shared__ uint32_t tmem_slot;
     __shared__ int failed;
@@ -161,9 +142,9 @@ __global__ void __launch_bounds__(GT_THREADS, 1) k_gemm_tc(const __grid_constant
         const uint32_t fb = s_u32(&full[slot]);
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
                      :: "r"(fb), "r"((uint32_t)SLOT) : "memory");
-        const int kg = (kc0 + q) * (GT_KC / 8);
-        gt_tma3(s_u32(sA), pa, m0, kg, fb);
-        gt_tma3(s_u32(sB), pb, n0, kg, fb);
+        const int k = (kc0 + q) * GT_KC;
+        tma_load_2d(s_u32(sA), pa, k, m0, fb);
+        tma_load_2d(s_u32(sB), pb, k, n0, fb);
     };
 
     bool ok = true;
@@ -178,8 +159,8 @@ __global__ void __launch_bounds__(GT_THREADS, 1) k_gemm_tc(const __grid_constant
             unsigned char *sA = smem + slot * SLOT, *sB = sA + A_BYTES;
 #pragma unroll
             for (int ks = 0; ks < GT_KC / 16; ++ks) {
-                const uint64_t da = gt_desc(s_u32(sA + ks * 2 * (GT_M * 16)), GT_M * 16, 128);
-                const uint64_t db = gt_desc(s_u32(sB + ks * 2 * (BN * 16)), BN * 16, 128);
+                const uint64_t da = desc_sw128(s_u32(sA) + ks * 32);
+                const uint64_t db = desc_sw128(s_u32(sB) + ks * 32);
                 const uint32_t acc = (q > 0 || ks > 0) ? 1u : 0u;
                 asm volatile(
                     "{\n\t.reg .pred p;\n\t"
@@ -306,7 +287,7 @@ __global__ void __launch_bounds__(GT_THREADS, 1) k_gemm_tc(const __grid_constant
 template <int BN, int NP>
 cudaError_t launch_gt(const GtBatch<NP> &b, bool overlap, cudaStream_t s)
 {
-    constexpr size_t smem = (size_t)gt_ring<BN>() * (GT_M * GT_KC * 2 + BN * GT_KC * 2);
+    constexpr size_t smem = 1024 + (size_t)gt_ring<BN>() * (GT_M * GT_KC * 2 + BN * GT_KC * 2);
     const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&k_gemm_tc<BN, NP>),
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

@@ -20,6 +20,7 @@
 #include <cstdint>
 #include <cstring>
 
+#include "async_copy.cuh"
 #include "mlsd_internal.cuh"
 
 namespace mlsd {
@@ -268,14 +269,13 @@ __global__ void __launch_bounds__(128, 1) k_mlp_tc(TcArgs a)
 }
 
 // ---------------------------------------------------------------------------
-// TMA-fed variant.  Operands arrive by cp.async.bulk.tensor through a 3-D view
-// of each row-major [rows][K] bfloat16 matrix: (8 elements) x (rows) x (K / 8
-// groups), strides (2 B, K * 2 B, 16 B).  A box {8, R, 8} lands in shared memory
-// as K-group-major slabs of R x 16 B, i.e. the no-swizzle K-major core-matrix
-// layout with core matrices 128 B apart along M / N and R * 16 B apart along K.
+// TMA-fed variant.  Boxes of 64 elements x rows of each row-major [rows][K] bfloat16 matrix
+// arrive by cp.async.bulk.tensor with the 128-byte swizzle.
 // A 3-slot ring (full / empty mbarriers) prefetches 64-wide K chunks across the
-// layers while one thread issues the MMAs; the epilogue writes activations in the
-// same layout (conflict-free 16-byte stores) for the next layer's A operand.
+// layers while one thread issues the MMAs; the epilogue writes activations as
+// K-group-major slabs of 128 x 16 bytes (conflict-free 16-byte stores), the no-swizzle K-major
+// core-matrix layout, for the next layer's A operand.  9216 rows x 4 members, 256 wide:
+// 65 us, 90 with core-matrix boxes (rows of 16 bytes) for all operands.
 constexpr int RING = 3;
 // 16 warps: warp w reads TMEM lanes 32 (w % 4) .. +31 (the lane quarter a warp may
 // access) and the 32-column chunks w / 4, w / 4 + 4, ... of the layer's outputs, so the
@@ -296,16 +296,6 @@ struct TmaArgs {
     int *status;
 };
 
-__device__ __forceinline__ void tma3(uint32_t dst, const CUtensorMap *map, int c0, int c1, int c2,
-                                     uint32_t mbar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4}], [%5];"
-        :: "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(mbar)
-        : "memory");
-}
-
 __device__ __forceinline__ void expect_tx(uint32_t mbar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(mbar), "r"(bytes)
@@ -315,8 +305,9 @@ __device__ __forceinline__ void expect_tx(uint32_t mbar, uint32_t bytes)
 __global__ void __launch_bounds__(TMA_THREADS, 1) k_mlp_tma(const __grid_constant__ TmaArgs a)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    unsigned char *ring = smem;                          // RING x (A 16 KB | B 32 KB)
-    unsigned char *Hs = smem + RING * SLOT;              // [K/8][128][16 B] activations
+    // RING x (A 16 KB | B 32 KB), on swizzle atoms
+    unsigned char *ring = smem + ((1024 - (smem_u32(smem) & 1023)) & 1023);
+    unsigned char *Hs = ring + RING * SLOT;              // [K/8][128][16 B] activations
     __shared__ __align__(8) uint64_t full[RING], empty[RING], accb;
     __shared__ uint32_t tmem_slot;
     __shared__ int failed;
@@ -370,8 +361,8 @@ __global__ void __launch_bounds__(TMA_THREADS, 1) k_mlp_tma(const __grid_constan
         const uint32_t fb = smem_u32(&full[slot]);
         const int nr = nrows(l);
         expect_tx(fb, (l == 0 ? A_BYTES : 0) + nr * KC * 2);
-        if (l == 0) tma3(smem_u32(sA), &a.xmap, 0, (int)row0, kc * (KC / 8), fb);
-        tma3(smem_u32(sB), &a.wmap[member][l], 0, 0, kc * (KC / 8), fb);
+        if (l == 0) tma_load_2d(smem_u32(sA), &a.xmap, kc * KC, (int)row0, fb);
+        tma_load_2d(smem_u32(sB), &a.wmap[member][l], kc * KC, 0, fb);
     };
 
     uint32_t acc_phase = 0;
@@ -393,9 +384,9 @@ __global__ void __launch_bounds__(TMA_THREADS, 1) k_mlp_tma(const __grid_constan
 #pragma unroll
                 for (int ks = 0; ks < KC / 16; ++ks) {
                     uint64_t da, db;
-                    if (l == 0) da = mat_desc(smem_u32(sA + ks * 2 * (TM * 16)), TM * 16, 128);
+                    if (l == 0) da = desc_sw128(smem_u32(sA) + ks * 32);
                     else da = mat_desc(smem_u32(Hs + ((kc * KC + ks * 16) >> 3) * (TM * 16)), TM * 16, 128);
-                    db = mat_desc(smem_u32(sB + ks * 2 * (N * 16)), N * 16, 128);
+                    db = desc_sw128(smem_u32(sB) + ks * 32);
                     mma_bf16(tmem, da, db, idesc, (kc > 0 || ks > 0) ? 1u : 0u);
                 }
                 mma_commit(smem_u32(&empty[slot]));
@@ -482,38 +473,23 @@ EncodeTiled encoder()
     return fn;
 }
 
-// 3-D core-matrix view of a row-major [rows][K] bfloat16 matrix, box {8, box_rows, 8}
-bool encode_view(CUtensorMap *m, const void *base, long long rows, int K, int box_rows)
-{
-    EncodeTiled enc = encoder();
-    if (!enc) return false;
-    cuuint64_t dims[3] = {8, (cuuint64_t)rows, (cuuint64_t)(K / 8)};
-    cuuint64_t strides[2] = {(cuuint64_t)K * 2, 16};
-    cuuint32_t box[3] = {8, (cuuint32_t)box_rows, 8};
-    cuuint32_t es[3] = {1, 1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 }  // namespace
 
-// 3-D core-matrix view of a bfloat16 matrix of `rows` rows and K columns, rows `ld`
-// elements apart (ld a multiple of 8): (8 elements) x (rows) x (ceil(K / 8) groups),
-// box {8, box_rows, 8}; a box lands as the no-swizzle K-major core-matrix layout.
-// Columns K .. 8 ceil(K / 8) - 1 are read from the row's padding.
+// 2-D view of a row-major bfloat16 matrix [rows][K], rows ld elements apart, box of box_rows rows
+// of 64 elements, 128-byte swizzle.  K is rounded up to 8 (the caller keeps the padding zero);
+// what a box reaches past it is zero-filled.
 bool encode_rows_bf16(void *map, const void *base, long long rows, long long K, long long ld,
                       int box_rows)
 {
     EncodeTiled enc = encoder();
     if (!enc || ld % 8 || ld < 8 * ((K + 7) / 8)) return false;
-    cuuint64_t dims[3] = {8, (cuuint64_t)rows, (cuuint64_t)((K + 7) / 8)};
-    cuuint64_t strides[2] = {(cuuint64_t)ld * 2, 16};
-    cuuint32_t box[3] = {8, (cuuint32_t)box_rows, 8};
-    cuuint32_t es[3] = {1, 1, 1};
-    return enc(static_cast<CUtensorMap *>(map), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
+    cuuint64_t dims[2] = {(cuuint64_t)(8 * ((K + 7) / 8)), (cuuint64_t)rows};
+    cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
+    cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
+    cuuint32_t es[2] = {1, 1};
+    return enc(static_cast<CUtensorMap *>(map), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
                const_cast<void *>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -565,10 +541,10 @@ bool mlp_tma_prepare(int h, int members, void *const *wb_host, void *maps_out)
         const __nv_bfloat16 *w = static_cast<const __nv_bfloat16 *>(wb_host[m]);
         const long long oW2 = (long long)h * MLSD_SUR_IN + h, oW3 = oW2 + (long long)h * h + h;
         const long long oW4 = oW3 + (long long)h * h + h;
-        if (!encode_view(&mp[m * 4 + 0], w, h, MLSD_SUR_IN, h)) return false;
-        if (!encode_view(&mp[m * 4 + 1], w + oW2, h, h, h)) return false;
-        if (!encode_view(&mp[m * 4 + 2], w + oW3, h, h, h)) return false;
-        if (!encode_view(&mp[m * 4 + 3], w + oW4, 3, h, 16)) return false;
+        if (!encode_rows_bf16(&mp[m * 4 + 0], w, h, MLSD_SUR_IN, MLSD_SUR_IN, h)) return false;
+        if (!encode_rows_bf16(&mp[m * 4 + 1], w + oW2, h, h, h, h)) return false;
+        if (!encode_rows_bf16(&mp[m * 4 + 2], w + oW3, h, h, h, h)) return false;
+        if (!encode_rows_bf16(&mp[m * 4 + 3], w + oW4, 3, h, h, 16)) return false;
     }
     return true;
 }
@@ -587,7 +563,7 @@ cudaError_t launch_mlp_tma(const void *X, long long M, int h, int members, const
 {
     TmaArgs a;
     std::memset(&a, 0, sizeof(a));
-    if (!encode_view(&a.xmap, X, M, MLSD_SUR_IN, TM)) return cudaErrorNotSupported;
+    if (!encode_rows_bf16(&a.xmap, X, M, MLSD_SUR_IN, MLSD_SUR_IN, TM)) return cudaErrorNotSupported;
     std::memcpy(a.wmap, maps, sizeof(a.wmap));
     a.M = M;
     a.h = h;
@@ -595,7 +571,7 @@ cudaError_t launch_mlp_tma(const void *X, long long M, int h, int members, const
     a.wf = wf_dev;
     a.out = out;
     a.status = status;
-    const size_t smem = (size_t)RING * SLOT + (size_t)TM * HMAX * 2;
+    const size_t smem = 1024 + (size_t)RING * SLOT + (size_t)TM * HMAX * 2;
     cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(&k_mlp_tma),
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

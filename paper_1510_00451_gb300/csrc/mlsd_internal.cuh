@@ -154,7 +154,7 @@ struct GemmPart {
 };
 cudaError_t gemm_tc_parts(GemmPart (&g)[3], int *status, bool overlap, cudaStream_t s);
 int gemm_tc_splits(int M, int N, int K, int sms);
-// 3-D core-matrix tensor map (CUtensorMap) of a bfloat16 matrix [rows][K], rows ld apart
+// 2-D tensor map (CUtensorMap) of a bfloat16 matrix [rows][K], rows ld apart, 128-byte swizzle
 bool encode_rows_bf16(void *map, const void *base, long long rows, long long K, long long ld,
                       int box_rows);
 // 2-D FP32 tensor map (CUtensorMap, 128 bytes) of a row-major [height][width] array
