@@ -1021,36 +1021,34 @@ __global__ void k_merge_fallback(int n, const int *n_dev, const int *idx, const 
     K[3 * p + 2] = b[2] + s[3];
 }
 
-// Transposes of row-major bfloat16 [rows][cols] (row stride cols) into [cols][ldT]:
-// dst[c][r] = src[r][c] for r < rows, zero for rows <= r < ldT.  32 x 32 tiles
-// through shared memory (reads and writes along rows); blockIdx.z picks the matrix.
-struct Transposes {
-    const __nv_bfloat16 *src[3];
-    __nv_bfloat16 *dst[3];
-    int rows[3], cols[3], ldT[3];
+// Transpose of a row-major bfloat16 [rows][cols] (row stride cols, cols even) into [cols][ldT]
+// (ldT even): dst[c][r] = src[r][c] for r < rows, zero for rows <= r < ldT.  Tile `tile` of 64 x 64
+// by 256 threads, two elements a load and store.
+struct Transpose {
+    const __nv_bfloat16 *src;
+    __nv_bfloat16 *dst;
+    int rows, cols, ldT, tiles;
 };
-__global__ void k_transpose_bf16(Transposes a)
+__device__ void transpose_tile(const Transpose &a, int tile, __nv_bfloat162 (*t)[33])
 {
-    __shared__ __nv_bfloat16 t[32][33];
-    chain_wait();
-    const int z = blockIdx.z, rows = a.rows[z], cols = a.cols[z], ldT = a.ldT[z];
-    const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-    if (r0 >= rows || c0 >= cols) return;
-    const __nv_bfloat16 *src = a.src[z];
-    __nv_bfloat16 *dst = a.dst[z];
+    const int tx = (a.cols + 63) / 64, r0 = tile / tx * 64, c0 = tile % tx * 64;
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int k = threadIdx.y + 8 * q;
-        const int r = r0 + k, c = c0 + threadIdx.x;
-        t[k][threadIdx.x] = (r < rows && c < cols) ? src[(long long)r * cols + c]
-                                                   : __float2bfloat16_rn(0.f);
+    for (int q = 0; q < 8; ++q) {
+        const int r = r0 + y + 8 * q, c = c0 + 2 * x;
+        t[y + 8 * q][x] = r < a.rows && c < a.cols
+                              ? *reinterpret_cast<const __nv_bfloat162 *>(a.src + (long long)r * a.cols + c)
+                              : __floats2bfloat162_rn(0.f, 0.f);
     }
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int k = threadIdx.y + 8 * q;
-        const int c = c0 + k, r = r0 + threadIdx.x;
-        if (c < cols && r < ldT) dst[(long long)c * ldT + r] = t[threadIdx.x][k];
+    for (int q = 0; q < 8; ++q) {
+        const int k = y + 8 * q, c = c0 + k, r = r0 + 2 * x;
+        if (c < a.cols && r < a.ldT) {
+            const __nv_bfloat162 lo = t[2 * x][k >> 1], hi = t[2 * x + 1][k >> 1];
+            *reinterpret_cast<__nv_bfloat162 *>(a.dst + (long long)c * a.ldT + r) =
+                (k & 1) ? __nv_bfloat162(lo.y, hi.y) : __nv_bfloat162(lo.x, hi.x);
+        }
     }
 }
 
@@ -1097,74 +1095,92 @@ __global__ void k_out_fwd(int M, int h, const __nv_bfloat16 *A3, const __nv_bflo
     }
 }
 
-// Partial sums of dW4[j][k] = sum_m dZ4[m][j] A3[m][k] and db4[j] = sum_m dZ4[m][j] over
-// the row chunk blockIdx.y (rows y*chunk .. +chunk-1): a block of 32 columns x 8 row groups
-// (rows g, g + 8, ...), reduced over the groups in order, into part[y][j][k] and (the
-// blocks of the first column tile) bpart[y][j]; k_grad_reduce adds the chunks in order
-__global__ void k_out_bwd_w(int M, int h, int chunk, const float *dZ4, const __nv_bfloat16 *A3,
-                            float *part, float *bpart)
+// What the backward pass needs after the loss, side by side in one launch:
+//   blocks [0, xblocks): dZ3 = bf16((dZ4 W4) gelu'(Z3)) into bfloat16 [M][h] and its transpose
+//     [h][ldT] (zero for M <= m < ldT), 32 x 32 tiles through shared memory;
+//   the next wblocks: partial sums of dW4[j][k] = sum_m dZ4[m][j] A3[m][k] and
+//     db4[j] = sum_m dZ4[m][j] over chunk y of the rows: 32 columns x 8 row groups (rows g,
+//     g + 8, ...), reduced over the groups in order, into part[y][j][k] and (the blocks of the
+//     first column tile) bpart[y][j]; k_grad_reduce adds the chunks in order;
+//   the rest: the transposes that the GEMMs after it read.
+struct OutBwd {
+    int M, h, chunk, ldT, xtiles, xblocks, wblocks;      // xtiles: tiles along h
+    const float *dZ4, *Z3;
+    const __nv_bfloat16 *A3, *W4;
+    __nv_bfloat16 *dZ, *dZT;
+    float *part, *bpart;
+    Transpose tr[3];
+};
+__global__ void __launch_bounds__(256) k_out_bwd(OutBwd a)
 {
-    __shared__ float red[8][4][33];
+    __shared__ __align__(16) unsigned char sm[64 * 33 * 4];
     chain_wait();
-    const int c = threadIdx.x & 31, g = threadIdx.x >> 5, k = blockIdx.x * 32 + c;
-    const int mb = blockIdx.y * chunk, me = min(M, mb + chunk);
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, b = 0.f;
-#pragma unroll 16
-    for (int m = mb + g; m < me; m += 8) {
-        const float x = k < h ? __bfloat162float(A3[(long long)m * h + k]) : 0.f;
-        const float d0 = dZ4[3 * m], d1 = dZ4[3 * m + 1], d2 = dZ4[3 * m + 2];
-        s0 = fmaf(d0, x, s0);
-        s1 = fmaf(d1, x, s1);
-        s2 = fmaf(d2, x, s2);
-        if (c < 3) b += c == 0 ? d0 : (c == 1 ? d1 : d2);
-    }
-    red[g][0][c] = s0; red[g][1][c] = s1; red[g][2][c] = s2; red[g][3][c] = b;
-    __syncthreads();
-    if (g < 3 && k < h) {
-        float t = 0.f;
-        for (int q = 0; q < 8; ++q) t += red[q][g][c];
-        part[((long long)blockIdx.y * 3 + g) * h + k] = t;
-    }
-    if (blockIdx.x == 0 && g == 3 && c < 3) {
-        float t = 0.f;
-        for (int q = 0; q < 8; ++q) t += red[q][3][c];
-        bpart[blockIdx.y * 3 + c] = t;
-    }
-}
-
-// dZ3 = bf16((dZ4 W4) gelu'(Z3)) into bfloat16 [M][h] and its transpose [h][ldT] (zero
-// for M <= m < ldT): 32 x 32 tiles through shared memory
-__global__ void k_out_bwd_x(int M, int h, const float *dZ4, const __nv_bfloat16 *W4, const float *Z3,
-                            __nv_bfloat16 *dZ, __nv_bfloat16 *dZT, int ldT)
-{
-    __shared__ __nv_bfloat16 t[32][33];
-    chain_wait();
-    const int m0 = blockIdx.y * 32, k0 = blockIdx.x * 32, k = k0 + threadIdx.x;
-    float w0 = 0.f, w1 = 0.f, w2 = 0.f;
-    if (k < h) {
-        w0 = __bfloat162float(W4[k]); w1 = __bfloat162float(W4[h + k]); w2 = __bfloat162float(W4[2 * h + k]);
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int q = threadIdx.y + 8 * i;
-        const int m = m0 + q;
-        __nv_bfloat16 v = __float2bfloat16_rn(0.f);
-        if (m < M && k < h) {
-            float d = dZ4[3 * m] * w0;
-            d = fmaf(dZ4[3 * m + 1], w1, d);
-            d = fmaf(dZ4[3 * m + 2], w2, d);
-            v = __float2bfloat16_rn(d * gelu_d(Z3[(long long)m * h + k]));
-            dZ[(long long)m * h + k] = v;
+    const int M = a.M, h = a.h, c = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const float *dZ4 = a.dZ4;
+    int blk = blockIdx.x;
+    if (blk < a.xblocks) {
+        auto t = reinterpret_cast<__nv_bfloat16 (*)[33]>(sm);
+        const int m0 = blk / a.xtiles * 32, k0 = blk % a.xtiles * 32, k = k0 + c;
+        float w0 = 0.f, w1 = 0.f, w2 = 0.f;
+        if (k < h) {
+            w0 = __bfloat162float(a.W4[k]);
+            w1 = __bfloat162float(a.W4[h + k]);
+            w2 = __bfloat162float(a.W4[2 * h + k]);
         }
-        t[q][threadIdx.x] = v;
-    }
-    __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int q = threadIdx.y + 8 * i;
-        const int kk = k0 + q, m = m0 + threadIdx.x;
-        if (kk < h && m < ldT) dZT[(long long)kk * ldT + m] = t[threadIdx.x][q];
+        for (int i = 0; i < 4; ++i) {
+            const int q = g + 8 * i, m = m0 + q;
+            __nv_bfloat16 v = __float2bfloat16_rn(0.f);
+            if (m < M && k < h) {
+                float d = dZ4[3 * m] * w0;
+                d = fmaf(dZ4[3 * m + 1], w1, d);
+                d = fmaf(dZ4[3 * m + 2], w2, d);
+                v = __float2bfloat16_rn(d * gelu_d(a.Z3[(long long)m * h + k]));
+                a.dZ[(long long)m * h + k] = v;
+            }
+            t[q][c] = v;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int q = g + 8 * i, kk = k0 + q, m = m0 + c;
+            if (kk < h && m < a.ldT) a.dZT[(long long)kk * a.ldT + m] = t[c][q];
+        }
+        return;
     }
+    blk -= a.xblocks;
+    if (blk < a.wblocks) {
+        auto red = reinterpret_cast<float (*)[4][33]>(sm);
+        const int bx = blk % a.xtiles, by = blk / a.xtiles, k = bx * 32 + c;
+        const int mb = by * a.chunk, me = min(M, mb + a.chunk);
+        float s0 = 0.f, s1 = 0.f, s2 = 0.f, b = 0.f;
+#pragma unroll 16
+        for (int m = mb + g; m < me; m += 8) {
+            const float x = k < h ? __bfloat162float(a.A3[(long long)m * h + k]) : 0.f;
+            const float d0 = dZ4[3 * m], d1 = dZ4[3 * m + 1], d2 = dZ4[3 * m + 2];
+            s0 = fmaf(d0, x, s0);
+            s1 = fmaf(d1, x, s1);
+            s2 = fmaf(d2, x, s2);
+            if (c < 3) b += c == 0 ? d0 : (c == 1 ? d1 : d2);
+        }
+        red[g][0][c] = s0; red[g][1][c] = s1; red[g][2][c] = s2; red[g][3][c] = b;
+        __syncthreads();
+        if (g < 3 && k < h) {
+            float t = 0.f;
+            for (int q = 0; q < 8; ++q) t += red[q][g][c];
+            a.part[((long long)by * 3 + g) * h + k] = t;
+        }
+        if (bx == 0 && g == 3 && c < 3) {
+            float t = 0.f;
+            for (int q = 0; q < 8; ++q) t += red[q][3][c];
+            a.bpart[by * 3 + c] = t;
+        }
+        return;
+    }
+    blk -= a.wblocks;
+    int z = 0;
+    while (z < 2 && blk >= a.tr[z].tiles) blk -= a.tr[z++].tiles;
+    transpose_tile(a.tr[z], blk, reinterpret_cast<__nv_bfloat162 (*)[33]>(sm));
 }
 
 // The gradient from its parts, one launch.  Blocks of the hidden layers' weights: dW_l = the K
@@ -1389,9 +1405,9 @@ cudaError_t sur_grad(int h, int M, const void *X, const float *Y, const float *w
 // then the weight gradients dW_l = dZ_l^T A_{l-1} of all three layers in one launch (K = the
 // batch, split over CTAs) and one launch that adds the partials in a fixed order and sums the
 // bias gradients.  dZ of the hidden layers is a bfloat16 operand throughout (the oracle's
-// emulation rounds it the same).  What bounds it is the chain of launches, so there are 11 of
+// emulation rounds it the same).  What bounds it is the chain of launches, so there are 9 of
 // them (25 when every small step had its own), each starting while its predecessor runs: h = 256,
-// 2048 rows 196 -> 115 us a gradient (131 before the swizzled operand copies).
+// 2048 rows 196 -> 100 us a gradient (116 with 11 launches).
 cudaError_t sur_grad_tc(int h, int M, const void *X, const float *Y, const float *wf,
                         const void *wb_, float *Z[4], void *Aact[3], float *dA, float *g,
                         double *part, double *loss_dev, float *ws, const SurTc &tc, int *status,
@@ -1401,38 +1417,44 @@ cudaError_t sur_grad_tc(int h, int M, const void *X, const float *Y, const float
     const __nv_bfloat16 *wb = static_cast<const __nv_bfloat16 *>(wb_);
     const int ldT = tc.ldT;
     if (M > tc.max_rows || ldT < ((M + 7) / 8) * 8) return cudaErrorInvalidValue;
-    const dim3 tb(32, 8);
-    // W_1^T, W_2^T for the data gradients, X^T for the first layer's weight gradient
-    Transposes tr;
-    for (int i = 0; i < 2; ++i) {
-        tr.src[i] = wb + L.w[i + 1]; tr.dst[i] = tc.WT[i];
-        tr.rows[i] = tr.cols[i] = tr.ldT[i] = h;
-    }
-    tr.src[2] = static_cast<const __nv_bfloat16 *>(X); tr.dst[2] = tc.XT;
-    tr.rows[2] = M; tr.cols[2] = MLSD_SUR_IN; tr.ldT[2] = ldT;
-    count_launches(5);
-    k_transpose_bf16<<<dim3((unsigned)((std::max(h, MLSD_SUR_IN) + 31) / 32),
-                            (unsigned)((std::max(h, M) + 31) / 32), 3), tb, 0, s>>>(tr);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = cudaSuccess;
+    count_launches(3);
     // forward, hidden layers on the tensor cores
     const __nv_bfloat16 *in = static_cast<const __nv_bfloat16 *>(X);
     for (int l = 0; l < 3 && e == cudaSuccess; ++l) {
         e = gemm_tc(0, M, h, L.din[l], in, L.din[l], wb + L.w[l], L.din[l], wf + L.b[l], Z[l],
-                    nullptr, Aact[l], tc.AT[l], ldT, status, true, s);
+                    nullptr, Aact[l], tc.AT[l], ldT, status, l > 0, s);
         in = static_cast<const __nv_bfloat16 *>(Aact[l]);
     }
     if (e != cudaSuccess) return e;
-    // output layer (3 outputs), loss and dZ4; partials of dW4 and db4; dZ_2 and its transpose
+    // output layer (3 outputs), loss and dZ4
     const int nloss = (M + 7) / 8, S = std::min(SPLIT_MAX, (M + 127) / 128), chunk = (M + S - 1) / S;
     float *opart = ws + 3 * sur_split_workspace(h), *obpart = opart + (long long)S * 3 * h;
     e = launch_chained(k_out_fwd, dim3((unsigned)nloss), 256, 0, true, s, M, h, in, wb + L.w[3],
                        wf + L.b[3], Y, Z[3], dA, part);
-    if (e == cudaSuccess)
-        e = launch_chained(k_out_bwd_w, dim3((unsigned)((h + 31) / 32), (unsigned)S), 256, 0, true, s, M, h,
-                           chunk, dA, in, opart, obpart);
-    if (e == cudaSuccess)
-        e = launch_chained(k_out_bwd_x, dim3((unsigned)((h + 31) / 32), (unsigned)((M + 31) / 32)), tb, 0,
-                           true, s, M, h, dA, wb + L.w[3], Z[2], tc.dZ[0], tc.dZT[2], ldT);
+    if (e != cudaSuccess) return e;
+    // partials of dW4 and db4; dZ_2 and its transpose; W_1^T, W_2^T for the data gradients and X^T
+    // for the first layer's weight gradient
+    OutBwd ob;
+    ob.M = M; ob.h = h; ob.chunk = chunk; ob.ldT = ldT;
+    ob.xtiles = (h + 31) / 32;
+    ob.xblocks = ob.xtiles * ((M + 31) / 32);
+    ob.wblocks = ob.xtiles * S;
+    ob.dZ4 = dA; ob.Z3 = Z[2]; ob.A3 = in; ob.W4 = wb + L.w[3];
+    ob.dZ = tc.dZ[0]; ob.dZT = tc.dZT[2];
+    ob.part = opart; ob.bpart = obpart;
+    int blocks = ob.xblocks + ob.wblocks;
+    for (int i = 0; i < 3; ++i) {
+        Transpose &t = ob.tr[i];
+        t.src = i < 2 ? wb + L.w[i + 1] : static_cast<const __nv_bfloat16 *>(X);
+        t.dst = i < 2 ? tc.WT[i] : tc.XT;
+        t.rows = i < 2 ? h : M;
+        t.cols = i < 2 ? h : MLSD_SUR_IN;
+        t.ldT = i < 2 ? h : ldT;
+        t.tiles = ((t.rows + 63) / 64) * ((t.cols + 63) / 64);
+        blocks += t.tiles;
+    }
+    e = launch_chained(k_out_bwd, dim3((unsigned)blocks), 256, 0, true, s, ob);
     // dZ_{l-1} = bf16((dZ_l W_l) gelu'(Z_{l-1})): A = dZ_l [M][h], B = W_l^T [din][h]
     for (int l = 2; l >= 1 && e == cudaSuccess; --l)
         e = gemm_tc(1, M, L.din[l], h, tc.dZ[l & 1], h, tc.WT[l - 1], h, nullptr, nullptr, Z[l - 1],
@@ -1453,7 +1475,7 @@ cudaError_t sur_grad_tc(int h, int M, const void *X, const float *Y, const float
     }
     e = gemm_tc_parts(gp, status, true, s);
     if (e != cudaSuccess) return e;
-    int blocks = 0;
+    blocks = 0;
     rd.bblocks = (h + 7) / 8;
     for (int l = 0; l < 3; ++l) {
         rd.part[l] = gp[l].part; rd.slices[l] = gp[l].splits;
