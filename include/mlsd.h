@@ -429,7 +429,8 @@ int mlsd_check_wait_timeout(mlsd_levels *h, int which, void *cuda_stream);
  *   dt, nsteps  time step and number of steps (nsteps >= 0)
  *   mass_out    host [nsteps + 1] or NULL: H^2 * sum(U) after each step (FP64);
  *               when non-NULL the call blocks until the steps are done.
- * Allocates (stream-ordered) a device scratch of N*N reals plus the mass list. */
+ * Above 32^2 (FP64: 16^2) allocates, stream-ordered from the library's pool,
+ * five N*N arrays (face coefficients and a field); and the mass list. */
 int mlsd_macro_step(int n_macro, void *U_dev, int precision, const double *K_dev, double dt,
                     int nsteps, double *mass_out_host, void *cuda_stream);
 
@@ -463,10 +464,11 @@ int mlsd_grid_psi(int n_modes, const int32_t *k1, const int32_t *k2, const doubl
  * u_t = v.grad_h u + kappa Lap_h u with v from psi by central differences,
  * Heun's RK2, nsteps steps.  u_dev [nf][nf] float in place; u_tmp_dev is a
  * caller-provided work field of the same size.  nf a multiple of 128.
- * One fused launch per step; the kernel (per-tile CTAs staged by cp.async, or
- * persistent CTAs fed by tensor copies) is picked once per process by timing
- * each on the caller's grid (MLSD_DNS_TY = 64 | 32 | t32 | t32x2 | t64 | t32p pins
- * one).  The persistent kernels take tiles from a per-device queue: one DNS
+ * Grids up to 1024^2: four steps per launch, tiles with a halo ("k_dns_steps").
+ * Larger ones: one fused launch per step; the kernel (per-tile CTAs staged by
+ * cp.async, or persistent CTAs fed by tensor copies) is picked once per process by
+ * timing each on the caller's grid (MLSD_DNS_TY = 64 | 32 | t32 | t32x2 | t64 | t32p
+ * pins one, on all grids).  The persistent kernels take tiles from a per-device queue: one DNS
  * run at a time per device.  Asynchronous: a tile copy that never lands (a
  * wait of about a second runs out) is reported by mlsd_dns_status.           */
 int mlsd_dns_run(int nf, float *u_dev, float *u_tmp_dev, const float *psi_dev, double kappa,
@@ -477,15 +479,16 @@ int mlsd_dns_run(int nf, float *u_dev, float *u_tmp_dev, const float *psi_dev, d
  * clears the flag.  MLSD_ECUDA if the stream reports an error.               */
 int mlsd_dns_status(void *cuda_stream);
 
-/* Name of the DNS kernel this process picked for mlsd_dns_run ("" before the
- * first run), e.g. "k_dns_tma<32,1>": static storage, not to be freed.      */
+/* Name of the DNS kernel of the last mlsd_dns_run ("" before the
+ * first run), e.g. "k_dns_tma<32,1>" or "k_dns_steps": static storage, not to be freed.      */
 const char *mlsd_dns_kernel(void);
 
 /* The direct simulation with the Sec. 4 boundary conditions (Dirichlet in x1,
  * periodic in x2), posed on [0, 2 pi] x [0, 2 pi) as mlsd_macro_step_dirichlet:
  * column 0 of u_dev is set to u_left and held, the virtual column nf has the
- * value u_right; psi (and so v) stays periodic.  One launch per RK stage (the
- * paper's 512 x 512 reference, L2-resident); any nf >= 4.
+ * value u_right; psi (and so v) stays periodic.  FP32: four steps per launch;
+ * FP64: a step per launch, from face coefficients formed once per run in a
+ * stream-ordered scratch of 2 nf^2 doubles; any nf >= 4.
  *   u_dev, u_tmp_dev  device [nf][nf], float (MLSD_FP32) or double (MLSD_FP64);
  *                     u_tmp_dev is a caller-provided work field
  *   psi_dev           device [nf][nf] float (mlsd_grid_psi)

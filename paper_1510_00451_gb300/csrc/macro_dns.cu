@@ -796,6 +796,8 @@ k_dns_steps(int nf, const float *uin, const float *__restrict__ psi, float *uout
 // 5 operations a cell and stage, none of them a conversion (aE and aN come from arrays formed
 // once per run; 12 operations and 4 conversions a cell and stage before).  512^2: 9.8 us a step
 // against 24.7 with a launch per stage.  The boundary values enter the first stage scaled by sqrt2.
+// Grids above kDirCoefMax^2 (1 GB of coefficients), and calls whose coefficients find no memory,
+// form them again in every step: 10 operations and 4 conversions more per cell.
 __global__ void k_dns_dir_coef(int nf, const float *__restrict__ psi, double cA, double d,
                                double *__restrict__ aE, double *__restrict__ aN)
 {
@@ -815,7 +817,8 @@ constexpr int kD64R = 2, kD64TX = 28;
 template <int TY>
 __global__ void __launch_bounds__(32 * (TY + 4) / kD64R)
 k_dns_dir_step64(int nf, const double *uin, double *uout, const double *__restrict__ aEg,
-                 const double *__restrict__ aNg, double d, double ul, double ur, double ul_s, double ur_s)
+                 const double *__restrict__ aNg, const float *__restrict__ psi, double cA, double d,
+                 double ul, double ur, double ul_s, double ur_s)
 {
     constexpr int R = kD64R, EY = TY + 4;
     __shared__ double A[EY * 32], Bf[EY * 32];
@@ -828,9 +831,17 @@ k_dns_dir_step64(int nf, const double *uin, double *uout, const double *__restri
     double u[R], aE[R], aN[R], aW[R], aS[R], s[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const long long c = (long long)wrap(gy0 + r) * nf + gx;
-        aE[r] = aEg[c];
-        aN[r] = aNg[c];
+        const int gy = wrap(gy0 + r);
+        const long long row = (long long)gy * nf, c = row + gx;
+        if (aEg) {
+            aE[r] = aEg[c];
+            aN[r] = aNg[c];
+        } else {                                        // as k_dns_dir_coef
+            const int gp = gy + 1 == nf ? 0 : gy + 1, gm = gy == 0 ? nf - 1 : gy - 1;
+            const int ap = gx + 1 == nf ? 0 : gx + 1, am = gx == 0 ? nf - 1 : gx - 1;
+            aE[r] = fma(cA, (double)psi[(long long)gm * nf + gx] - (double)psi[(long long)gp * nf + gx], d);
+            aN[r] = fma(cA, (double)psi[row + ap] - (double)psi[row + am], d);
+        }
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) { aW[r] = two_d - aE[r]; aS[r] = two_d - aN[r]; }
@@ -1317,9 +1328,10 @@ cudaError_t launch_wait_check_tile(int *status, cudaStream_t s)
     return cudaGetLastError();
 }
 
+constexpr int kDirCoefMax = 8192;
 size_t dns_dirichlet_scratch_bytes(int nf, int precision, int nsteps)
 {
-    return precision == MLSD_FP64 && nsteps > 0 ? 2 * (size_t)nf * nf * sizeof(double) : 0;
+    return precision == MLSD_FP64 && nsteps > 0 && nf <= kDirCoefMax ? 2 * (size_t)nf * nf * sizeof(double) : 0;
 }
 
 cudaError_t dns_run_dirichlet(int nf, void *u, void *u_tmp, const float *psi, int precision,
@@ -1339,11 +1351,11 @@ cudaError_t dns_run_dirichlet(int nf, void *u, void *u_tmp, const float *psi, in
     if (precision != MLSD_FP64)
         return dns_multi<true>(nf, static_cast<float *>(u), static_cast<float *>(u_tmp), psi, (float)cA,
                                (float)cD, nsteps, (float)ul, (float)ur, s);
-    double *aE = static_cast<double *>(scratch), *aN = aE + (size_t)nf * nf;
+    double *aE = static_cast<double *>(scratch), *aN = aE ? aE + (size_t)nf * nf : nullptr;
     const double r2 = 0.70710678118654752440;
     const long long n2 = (long long)nf * nf;
-    count_launches(1 + (long long)nsteps);
-    k_dns_dir_coef<<<(unsigned)((n2 + 255) / 256), 256, 0, s>>>(nf, psi, r2 * cA, r2 * cD, aE, aN);
+    count_launches((aE ? 1 : 0) + (long long)nsteps);
+    if (aE) k_dns_dir_coef<<<(unsigned)((n2 + 255) / 256), 256, 0, s>>>(nf, psi, r2 * cA, r2 * cD, aE, aN);
     // tiles of 32 rows where they give every SM one, else of 8 (an SM's FP64 rate decides)
     const unsigned gx = (unsigned)((nf + kD64TX - 1) / kD64TX);
     const bool tall = (long long)gx * ((nf + 31) / 32) >= 152;
@@ -1353,8 +1365,8 @@ cudaError_t dns_run_dirichlet(int nf, void *u, void *u_tmp, const float *psi, in
     const double sq2 = 1.4142135623730951;
     double *a = static_cast<double *>(u), *b = static_cast<double *>(u_tmp);
     for (int k = 0; k < nsteps; ++k) {
-        const cudaError_t e = launch_chained(fn, grid, nt, 0, k > 0, s, nf, a, b, aE, aN, r2 * cD, ul, ur,
-                                             sq2 * ul, sq2 * ur);
+        const cudaError_t e = launch_chained(fn, grid, nt, 0, k > 0, s, nf, a, b, aE, aN, psi, r2 * cA,
+                                             r2 * cD, ul, ur, sq2 * ul, sq2 * ur);
         if (e != cudaSuccess) return e;
         std::swap(a, b);
     }

@@ -114,16 +114,20 @@ namespace {
 // the system at every synchronisation, and the next call maps it again (about 150 us a call);
 // the library's own pool, one per device, keeps up to kPoolKeep bytes.  mlsd_free_levels and
 // mlsd_surrogate_free give back what is idle.  The pool itself orders allocations and frees
-// between streams and threads.
+// between streams and threads.  Under capture the allocation belongs to the graph, and no pool may
+// be made: the default one.
 constexpr unsigned long long kPoolKeep = 32ull << 20;
 std::mutex g_pool_mu;
 std::map<int, cudaMemPool_t> g_pool;
 
 cudaError_t ws_alloc(void **p, size_t bytes, cudaStream_t s)
 {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s, &cs);
     if (e != cudaSuccess) return e;
+    if (cs != cudaStreamCaptureStatusNone) return cudaMallocAsync(p, bytes, s);
+    int dev = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     cudaMemPool_t pool = nullptr;
     {
         std::lock_guard<std::mutex> lock(g_pool_mu);
@@ -1364,7 +1368,10 @@ int mlsd_dns_run_dirichlet(int nf, void *u_dev, void *u_tmp_dev, const float *ps
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     const size_t sb = dns_dirichlet_scratch_bytes(nf, precision, nsteps);
     void *scratch = nullptr;
-    if (sb) CK(ws_alloc(&scratch, sb, s));
+    if (sb && ws_alloc(&scratch, sb, s) != cudaSuccess) {      // without it: slower, the same results
+        cudaGetLastError();
+        scratch = nullptr;
+    }
     const cudaError_t e = dns_run_dirichlet(nf, u_dev, u_tmp_dev, psi_dev, precision, kappa, dt, nsteps,
                                             u_left, u_right, scratch, s);
     if (scratch) cudaFreeAsync(scratch, s);

@@ -103,3 +103,56 @@ def test_box_averages_not_finite(mlsd, torch_mod, r):
     V = U.cpu().numpy()
     assert np.isnan(V[0, 0]) and V[1, 2] == -np.inf and np.isnan(V[1, 0])
     assert np.all(V[[0, 0, 1, 2, 2, 2], [1, 2, 1, 0, 1, 2]] == 1.0)
+
+
+def test_dirichlet_without_coefficients(mlsd, torch_mod):
+    # above 8192^2 the FP64 steps form their coefficients themselves: the same operations as on
+    # smaller grids.  psi and u do not depend on x2 (v2 = 0 exactly, v1 = 0), so each row is the
+    # heat equation of a 1-D row: the sum of the same five terms, some 10 roundings of O(1) values
+    nf, steps, dt, kappa = 8193, 2, 1e-8, 0.7
+    h = 2 * np.pi / nf
+    x = np.arange(nf) * h
+    row = np.cos(3 * x) + 1.5
+    u = torch_mod.tensor(row, dtype=torch_mod.float64, device="cuda:0").repeat(nf, 1).contiguous()
+    ut = torch_mod.empty_like(u)
+    psi = torch_mod.full((nf, nf), 0.25, dtype=torch_mod.float32, device="cuda:0")
+    mlsd.dns_run_dirichlet(u, ut, psi, kappa, dt, steps, 2.5, 2.5)
+    ref = row.copy()
+    ref[0] = 2.5
+
+    def f(v):
+        e = np.append(v, 2.5)
+        g = np.zeros_like(v)
+        g[1:] = kappa * (e[2:] - 2 * e[1:-1] + e[:-2]) / (h * h)
+        return g
+    for _ in range(steps):
+        k1 = f(ref)
+        ref = ref + dt / 2 * (k1 + f(ref + dt * k1))
+    got = u.cpu().numpy()
+    assert np.max(np.abs(got[[0, 1, 4000, nf - 1]] - ref)) <= 40 * 2.0**-52 * 2.5
+    assert np.array_equal(got[4000], got[17]) or np.max(np.abs(got[4000] - got[17])) <= 40 * 2.0**-52 * 2.5
+
+
+@pytest.mark.parametrize("nf,prec", [(512, "fp32"), (512, "fp64"), (2048, "fp32")])
+def test_captured_runs(mlsd, torch_mod, nf, prec):
+    # a captured run, replayed on new values of the same buffers, gives the direct call's bits
+    psi, _, dt = _flow(torch_mod, nf)
+    dtype = torch_mod.float64 if prec == "fp64" else torch_mod.float32
+    u0 = torch_mod.tensor(flows.gaussian_u0(nf), dtype=dtype, device="cuda:0")
+    u, ut = u0.clone(), torch_mod.empty_like(u0)
+
+    def step():
+        if prec == "fp64":
+            mlsd.dns_run_dirichlet(u, ut, psi, 1.0, dt, 5, 1.0, 0.0)
+        else:
+            mlsd.dns_run(u, ut, psi, 1.0, dt, 5)
+    step()
+    ref = u.clone()
+    u.copy_(u0)
+    g = torch_mod.cuda.CUDAGraph()
+    with torch_mod.cuda.graph(g):
+        step()
+    assert torch_mod.equal(u, u0)
+    g.replay()
+    torch_mod.cuda.synchronize()
+    assert torch_mod.equal(u, ref)
