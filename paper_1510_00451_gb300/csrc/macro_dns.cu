@@ -794,7 +794,7 @@ k_dns_steps(int nf, const float *uin, const float *__restrict__ psi, float *uout
 //   A' x = aE xE + aW xW + aN xN + aS xS - 4 d x,   d = dt kappa / (sqrt2 h^2),
 //   aE, aW = d +- c1, aN, aS = d +- c2,  c1, c2 = dt / (4 sqrt2 h^2) (psiS - psiN, psiE - psiW):
 // 5 operations a cell and stage, none of them a conversion (aE and aN come from arrays formed
-// once per run; 12 operations and 4 conversions a cell and stage before).  512^2: 9.8 us a step
+// once per run; 12 operations and 4 conversions a cell and stage before).  512^2: 8.9 us a step
 // against 24.7 with a launch per stage.  The boundary values enter the first stage scaled by sqrt2.
 // Grids above kDirCoefMax^2 (1 GB of coefficients), and calls whose coefficients find no memory,
 // form them again in every step: 10 operations and 4 conversions more per cell.
