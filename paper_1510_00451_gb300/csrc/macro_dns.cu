@@ -53,11 +53,11 @@ __device__ __forceinline__ real macro_face(int q, const double *Kg, int N, int i
     const int c = j * N + i;
     const int o = q < 2 ? j * N + (i + 1 == N ? 0 : i + 1) : (j + 1 == N ? 0 : j + 1) * N + i;
     const int k = q == 0 ? 0 : (q == 2 ? 2 : 1);
-    return ((q & 1) ? (real)0.25 * f : f) * ((real)Kg[3 * c + k] + (real)Kg[3 * o + k]);
+    return ((q & 1) ? (real)0.25 * f : f) * ((real)Kg[3LL * c + k] + (real)Kg[3LL * o + k]);
 }
 
-// coefficients into co [4][N][N]; U into V when V is given; with dir, column 0 of U (and V)
-// takes the boundary value ul
+// coefficients into co [4][N][N] (above 23170^2 cells they do not fit 32-bit indices); U into V when
+// V is given; with dir, column 0 of U (and V) takes the boundary value ul
 template <typename real>
 __global__ void k_macro_prep(int N, const double *Kg, real f, real *co, real *U, real *V, int dir,
                              real ul)
@@ -66,7 +66,7 @@ __global__ void k_macro_prep(int N, const double *Kg, real f, real *co, real *U,
     if (c >= NN) return;
     const int i = c % N, j = c / N;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) co[q * NN + c] = macro_face(q, Kg, N, i, j, f);
+    for (int q = 0; q < 4; ++q) co[(long long)q * NN + c] = macro_face(q, Kg, N, i, j, f);
     if (dir && i == 0) U[c] = ul;
     if (V) V[c] = (dir && i == 0) ? ul : U[c];
 }

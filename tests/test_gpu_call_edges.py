@@ -1,0 +1,49 @@
+"""Calls at the edges of what the entry points accept."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch_mod():
+    import torch
+    assert torch.cuda.is_available()
+    return torch
+
+
+@pytest.fixture(scope="module")
+def mlsd():
+    import paper_1510_00451_gb300 as m
+    return m
+
+
+def test_macro_past_32_bit_coefficients(mlsd, torch_mod):
+    # 4 N^2 > 2^31 - 1: the face coefficients of the last cells lie past a 32-bit index.  K and U
+    # depend on x1 only, so every row is the same 1-D problem: Heun in FP64 on the host against a few
+    # FP32 roundings of O(1) values
+    N, steps = 23171, 2
+    if torch_mod.cuda.mem_get_info()[0] < 40 << 30:
+        pytest.skip("needs 40 GB")
+    H = 2 * np.pi / N
+    x = np.arange(N) * H
+    k = 1.0 + 0.5 * np.cos(5 * x)
+    row = 1.5 + np.cos(3 * x)
+    dt = 0.1 * H * H
+    K = torch_mod.zeros(N, N, 3, dtype=torch_mod.float64, device="cuda:0")
+    K[:, :, 0] = torch_mod.tensor(k, device="cuda:0")
+    K[:, :, 2] = 0.75
+    U = torch_mod.tensor(row, dtype=torch_mod.float32, device="cuda:0").repeat(N, 1)
+    mlsd.macro_step(U, K, dt, steps, want_mass=False)
+    kf = 0.5 * (k + np.roll(k, -1)) * dt / (H * H)
+
+    def f(u):
+        flux = kf * (np.roll(u, -1) - u)
+        return flux - np.roll(flux, 1)
+    ref = row
+    for _ in range(steps):
+        s = ref + f(ref)
+        ref = 0.5 * (ref + s + f(s))
+    for j in (0, 1, N // 2, N - 2, N - 1):
+        assert np.abs(U[j].double().cpu().numpy() - ref).max() < 20 * 2.0**-24 * 2.5
+    assert torch_mod.equal(U[0], U[N - 1]) and bool((U == U[0]).all())
