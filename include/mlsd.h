@@ -306,7 +306,9 @@ int mlsd_surrogate_set_params(mlsd_surrogate *s, int member, const float *params
 int mlsd_surrogate_get_params(mlsd_surrogate *s, int member, float *params_host);
 /* Features of every patch of a level (one patch size per level, n = 32, 64,
  * 128 or 256; FP32) with base B_dev [P][3]: X_dev bfloat16 [P][640]; F32_dev
- * [P][606] or NULL.  Levels of several sizes: MLSD_EUNSUPPORTED.            */
+ * [P][606] or NULL; both may start at any element (pairs are stored where X_dev
+ * is 4-byte and F32_dev 8-byte aligned).  Levels of several sizes:
+ * MLSD_EUNSUPPORTED.                                                        */
 int mlsd_surrogate_features(mlsd_levels *h, int level, const double *B_dev, void *X_dev,
                             float *F32_dev, void *cuda_stream);
 /* Mean-squared-error loss of one member on M <= max_batch rows (X bfloat16

@@ -2,6 +2,8 @@
 import numpy as np
 import pytest
 
+from inputs import flows
+
 pytestmark = pytest.mark.gpu
 
 
@@ -47,3 +49,29 @@ def test_macro_past_32_bit_coefficients(mlsd, torch_mod):
     for j in (0, 1, N // 2, N - 2, N - 1):
         assert np.abs(U[j].double().cpu().numpy() - ref).max() < 20 * 2.0**-24 * 2.5
     assert torch_mod.equal(U[0], U[N - 1]) and bool((U == U[0]).all())
+
+
+@pytest.mark.parametrize("n", [32, 64])
+@pytest.mark.parametrize("xo,fo", [(1, 0), (0, 1), (3, 3), (2, 2)])
+def test_feature_rows_at_any_offset(mlsd, torch_mod, n, xo, fo):
+    # X and F32 need the alignment of their elements only
+    lv = mlsd.Levels(flows.cellular_two_scale(0.8, 0.5, 4), 0.03, 3, [1, 4, 8], [n, n],
+                     n_burn_fixed=0, n_avg_fixed=4)
+    B = torch_mod.tensor([[0.05, 0.01, 0.04]] * 9, dtype=torch_mod.float64, device="cuda:0")
+
+    def rows(xo, fo):
+        X = torch_mod.full((9 * mlsd.SUR_IN + 8,), -7.0, dtype=torch_mod.bfloat16, device="cuda:0")
+        F = torch_mod.full((9 * mlsd.SUR_FEATURES + 8,), -7.0, device="cuda:0")
+        x, f = X[xo:xo + 9 * mlsd.SUR_IN], F[fo:fo + 9 * mlsd.SUR_FEATURES]
+        lv.features(2, B, x, f)
+        outside = torch_mod.cat([X[:xo].float(), X[xo + len(x):].float(), F[:fo], F[fo + len(f):]])
+        assert bool((outside == -7.0).all())
+        return x.clone(), f.clone()
+    x0, f0 = rows(0, 0)
+    x1, f1 = rows(xo, fo)
+    assert torch_mod.equal(x0, x1) and torch_mod.equal(f0, f1)
+    # the data set's rows come from the same kernel
+    X = torch_mod.empty(9 * mlsd.SUR_IN + 8, dtype=torch_mod.bfloat16, device="cuda:0")[xo:xo + 9 * mlsd.SUR_IN]
+    Y = torch_mod.empty(9, 3, device="cuda:0")
+    lv.surrogate_dataset(2, B, X, Y)
+    assert torch_mod.equal(X, x0)
