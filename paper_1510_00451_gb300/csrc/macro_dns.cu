@@ -904,18 +904,19 @@ __global__ void k_dns_vmax(int nf, const float *psi, float ax, unsigned *out)
 // every node in FP64 took 8 times as long as reading it.  So up to T PER nodes at a time are
 // added as integers: with E the largest exponent of the n <= 2^bits nodes and shift = 38 - bits,
 // each becomes its 24-bit significand in units of 2^(E - 150 - shift), so that n of them fit
-// 62 bits.  Nodes within 2^shift (2^26 at least) of the largest are added exactly, smaller ones
-// rounded to the unit (2^-49 of the largest at most), and the sum is rounded once to FP64.
-// Infinities and NaN are added in FP64.  The 8 warps' FP64 work is left to one of them (a warp
+// 62 bits.  That is exact where every node but zeros is within 2^shift (2^26 at least) of the
+// largest, and the sum is rounded once to FP64.  Nodes further apart, which integers would round to
+// their unit, are added in FP64, as infinities and NaN are.  The 8 warps' FP64 work is left to one of them (a warp
 // with one box takes as long as one with 8).  8192^2 onto 64^2, 128^2, 512^2: 288, 367, 2081 us
-// for a CTA a box in FP64, 118, 122, 144 so (reading them once: 40).  What bounds it: the integer
-// operations, about 25 a node.
+// for a CTA a box in FP64; 130, 136, 150 so (118, 122, 144 without looking for nodes too far
+// apart, each of them then off by up to 2^-50 of the largest); 311, 314, 359 where every box has such
+// nodes (reading them once: 40).  What bounds it: the integer operations, about 27 a node.
 template <int W, int PER>
 __global__ void __launch_bounds__(256) k_coarse(int nf, const float *__restrict__ u, int N, float *U,
                                                 double *box, int bits)
 {
     constexpr int T = 32 * W, BOXES = 8 / W;          // threads per box, boxes per CTA
-    __shared__ unsigned tops[8];
+    __shared__ unsigned tops[8], lows[8];
     __shared__ long long accs[8];
     __shared__ double sums[8];
     const int r = nf / N, n = r * r, t = threadIdx.x % T, warp = threadIdx.x >> 5, w0 = warp / W * W;
@@ -923,12 +924,17 @@ __global__ void __launch_bounds__(256) k_coarse(int nf, const float *__restrict_
     const bool in = b < (long long)N * N;
     const int i = (int)(b % N), j = (int)(b / N), x0 = i * r - r / 2, y0 = j * r - r / 2;
     const int sx = T % r, sy = T / r, shift = 38 - bits;
+    auto exponent = [](unsigned a) { return max(1, (int)(a >> 23)); };    // denormals: that of 2^-126
+    // whether nodes of magnitudes low + 1 .. top (zeros aside) fit integers exactly
+    auto integers = [&](unsigned top, unsigned low) {
+        return exponent(top) < 255 && exponent(top) - exponent(low + 1) <= shift;
+    };
     // thread k < BOXES: the sum of the CTA's k-th box.  One chunk of nodes unless W = 8
     double total = 0.0;
     int x = t % r, y = t / r;
     for (int base = 0; base < (W < 8 ? 1 : n); base += T * PER) {
         // the lane's nodes: every T-th of the box's, row by row
-        unsigned v[PER], top = 0;
+        unsigned v[PER], top = 0, low = ~0u;              // low: the least magnitude - 1, zeros last
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
             int gx = x0 + x, gy = y0 + y;
@@ -940,24 +946,26 @@ __global__ void __launch_bounds__(256) k_coarse(int nf, const float *__restrict_
             if (x >= r) { x -= r; ++y; }
         }
 #pragma unroll
-        for (int k = 0; k < PER; ++k) top = max(top, v[k] & 0x7fffffffu);
+        for (int k = 0; k < PER; ++k) {
+            top = max(top, v[k] & 0x7fffffffu);
+            low = min(low, (v[k] & 0x7fffffffu) - 1u);
+        }
         top = __reduce_max_sync(0xffffffffu, top);
-        if ((threadIdx.x & 31) == 0) tops[warp] = top;
+        low = __reduce_min_sync(0xffffffffu, low);
+        if ((threadIdx.x & 31) == 0) { tops[warp] = top; lows[warp] = low; }
         if constexpr (W > 1) {
             __syncthreads();
 #pragma unroll
-            for (int w = 0; w < W; ++w) top = max(top, tops[w0 + w]);
+            for (int w = 0; w < W; ++w) { top = max(top, tops[w0 + w]); low = min(low, lows[w0 + w]); }
         }
-        const int E = max(1, (int)(top >> 23));        // denormals: the exponent of 2^-126
+        const int E = exponent(top);
         long long acc = 0;
-        if (E < 255) {
+        if (integers(top, low)) {
 #pragma unroll
             for (int k = 0; k < PER; ++k) {
                 const int e = (v[k] >> 23) & 255, sh = shift - (E - max(1, e));
                 const unsigned long long m = (v[k] & 0x7fffffu) | (e ? 0x800000u : 0u);
-                long long q = 0;
-                if (sh >= 0) q = (long long)(m << sh);
-                else if (sh > -25) q = (long long)((m + (1ull << (-sh - 1))) >> -sh);
+                const long long q = (long long)(m << (sh & 63));          // sh < 0 for zeros only
                 acc += (v[k] >> 31) ? -q : q;
             }
             for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -971,13 +979,15 @@ __global__ void __launch_bounds__(256) k_coarse(int nf, const float *__restrict_
         }
         __syncthreads();
         if (threadIdx.x < BOXES) {
-            unsigned tb = 0;
+            unsigned tb = 0, lb = ~0u;
             long long a = 0;
-            for (int w = 0; w < W; ++w) tb = max(tb, tops[threadIdx.x * W + w]);
-            const int Eb = max(1, (int)(tb >> 23));
-            if (Eb < 255) {
+            for (int w = 0; w < W; ++w) {
+                tb = max(tb, tops[threadIdx.x * W + w]);
+                lb = min(lb, lows[threadIdx.x * W + w]);
+            }
+            if (integers(tb, lb)) {
                 for (int w = 0; w < W; ++w) a += accs[threadIdx.x * W + w];
-                total += ldexp((double)a, Eb - 150 - shift);
+                total += ldexp((double)a, exponent(tb) - 150 - shift);
             } else {
                 for (int w = 0; w < W; ++w) total += sums[threadIdx.x * W + w];
             }

@@ -1,4 +1,6 @@
 """Calls at the edges of what the entry points accept."""
+import math
+
 import numpy as np
 import pytest
 
@@ -75,3 +77,39 @@ def test_feature_rows_at_any_offset(mlsd, torch_mod, n, xo, fo):
     Y = torch_mod.empty(9, 3, device="cuda:0")
     lv.surrogate_dataset(2, B, X, Y)
     assert torch_mod.equal(X, x0)
+
+
+@pytest.mark.parametrize("r", [4, 16, 32, 64, 100])
+@pytest.mark.parametrize("kind", ["one large", "cancelling", "spread", "denormal"])
+def test_box_sums_of_unequal_nodes(mlsd, torch_mod, r, kind):
+    # the box's sum in FP64: no worse than adding its nodes one by one in a tree of the kernel's
+    # depth (16 nodes a lane, 5 levels of a warp, 8 warps, a chunk after the other), each addition
+    # off by half a unit of the sum of the magnitudes at most
+    rng = np.random.default_rng(r)
+    u = np.full((r, r), 3e-15) * rng.uniform(0.5, 1.5, (r, r))
+    if kind == "one large":
+        u[r // 2, 1] = 1.0
+    if kind == "cancelling":
+        u[r // 2, 1], u[0, r - 1] = 1.0, -1.0
+    if kind == "spread":
+        u = rng.standard_normal((r, r)) * 10.0 ** rng.uniform(-30, 5, (r, r))
+    if kind == "denormal":
+        u = rng.standard_normal((r, r)) * 2.0 ** rng.uniform(-148, -60, (r, r))
+    u = u.astype(np.float32)
+    U = torch_mod.empty(1, 1, dtype=torch_mod.float32, device="cuda:0")
+    m = mlsd.coarse_grain(torch_mod.tensor(u, device="cuda:0"), 1, U)
+    exact, mag = math.fsum(u.ravel().astype(float)), math.fsum(np.abs(u.ravel().astype(float)))
+    depth = 16 + 5 + 8 + (r * r + 4095) // 4096
+    h2 = (2 * np.pi / r) ** 2
+    assert abs(m / h2 - exact) <= (depth + 4) * 2.0**-53 * mag
+    mean = exact / (r * r)
+    assert abs(float(U) - mean) <= abs(mean) * 2.0**-24 * 1.01 + depth * 2.0**-53 * mag / (r * r) + 2.0**-150
+    # whole boxes of the same kind beside narrow ones
+    v = np.tile(u, (3, 3))
+    v[:r, :r] = 0.5
+    V = torch_mod.empty(3, 3, dtype=torch_mod.float32, device="cuda:0")
+    v = np.roll(v, (-(r // 2), -(r // 2)), (0, 1))
+    mlsd.coarse_grain(torch_mod.tensor(v, device="cuda:0"), 3, V, want_mass=False)
+    V = V.cpu().numpy()
+    assert V[0, 0] == 0.5 and np.all(np.abs(V.ravel()[1:] - mean) <=
+                                     abs(mean) * 2.0**-24 * 1.01 + depth * 2.0**-53 * mag / (r * r) + 2.0**-150)
