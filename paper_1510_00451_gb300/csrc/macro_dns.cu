@@ -1128,33 +1128,37 @@ static cudaError_t dns_launch(int nf, const float *a, const float *psi, float *b
                           b, ax, kd, dt);
 }
 
-// the two tile counters of the persistent kernels, per device (zeroed once), and
-// which one the next launch on that device takes (every persistent launch, of any
-// tile shape, alternates them: each launch zeroes the other for its successor)
-static std::vector<int> g_dns_which;
-// the two tile counters of the persistent kernels, per device (zeroed once)
-static cudaError_t dns_queue(int dev, cudaStream_t s, int **out, int *which)
+// The two tile counters of the persistent kernels.  A run zeroes both before its first launch, then
+// its launches alternate them, each zeroing the other for its successor: a run does not depend on
+// what ran before it, so that a captured one can be replayed (the counters kept between runs by
+// the host were frozen into a graph: a replay could start on a used counter and leave tiles out).
+// The memset costs a run about 2 us, a step of these kernels takes 10 and more.
+struct DnsQueue {
+    int *counters = nullptr;
+    int which = 0;
+};
+static cudaError_t dns_queue(DnsQueue &out, cudaStream_t s)
 {
     static std::mutex mu;
-    static std::vector<int *> q;
-    std::lock_guard<std::mutex> lock(mu);
-    if ((int)q.size() <= dev) q.resize(dev + 1, nullptr);
-    if ((int)g_dns_which.size() <= dev) g_dns_which.resize(dev + 1, 0);
-    if (!q[dev]) {
-        cudaError_t e = cudaMalloc((void **)&q[dev], 2 * sizeof(int));
-        if (e == cudaSuccess) e = cudaMemsetAsync(q[dev], 0, 2 * sizeof(int), s);
+    static std::vector<int *> q;                    // by device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        if ((int)q.size() <= dev) q.resize(dev + 1, nullptr);
+        if (!q[dev]) e = cudaMalloc((void **)&q[dev], 2 * sizeof(int));
         if (e != cudaSuccess) { q[dev] = nullptr; return e; }
+        out.counters = q[dev];
     }
-    *out = q[dev];
-    *which = g_dns_which[dev];
-    g_dns_which[dev] ^= 1;
-    return cudaSuccess;
+    out.which = 0;
+    return cudaMemsetAsync(out.counters, 0, 2 * sizeof(int), s);
 }
 
 template <int DTY, int NBUF, bool PAIR = false>
 static cudaError_t dns_launch_tma(int nf, const CUtensorMap &ma, const CUtensorMap &mp,
                                   const float *a, const float *psi, float *b, float ax, float kd,
-                                  float dt, bool overlap, cudaStream_t s)
+                                  float dt, DnsQueue &queue, bool overlap, cudaStream_t s)
 {
     using T = DnsTma<DTY, NBUF>;
     constexpr int DTH = DnsTile<DTY>::DTH;
@@ -1180,11 +1184,10 @@ static cudaError_t dns_launch_tma(int nf, const CUtensorMap &ma, const CUtensorM
     }
     const long long ntiles = (long long)(nf / DTX) * (nf / DTY);
     const int grid = (int)std::min<long long>(ntiles, (long long)res * sms);
-    int *queue = nullptr, which = 0;                 // launches alternate the two counters
-    e = dns_queue(dev, s, &queue, &which);
-    if (e != cudaSuccess) return e;
+    const int which = queue.which;
+    queue.which ^= 1;
     return launch_chained(k_dns_tma<DTY, NBUF, PAIR>, dim3((unsigned)grid), DTH, T::SMEM, overlap, s, ma, mp, nf,
-                          a, psi, b, ax, kd, dt, queue, which);
+                          a, psi, b, ax, kd, dt, queue.counters, which);
 }
 
 // DNS kernel variants: per-tile CTAs staged by cp.async (tile height 64 rows, 2 CTAs/SM,
@@ -1198,16 +1201,16 @@ static int g_dns_kind = -1;
 
 static cudaError_t dns_launch_kind(int kind, int nf, const CUtensorMap *maps, int ia,
                                    const float *a, const float *psi, float *b, float ax, float kd,
-                                   float dt, bool overlap, cudaStream_t s)
+                                   float dt, DnsQueue &queue, bool overlap, cudaStream_t s)
 {
     switch (kind) {
     case kCp64: return dns_launch<64>(nf, a, psi, b, ax, kd, dt, overlap, s);
     case kCp32: return dns_launch<32>(nf, a, psi, b, ax, kd, dt, overlap, s);
-    case kTma32: return dns_launch_tma<32, 1>(nf, maps[ia], maps[2], a, psi, b, ax, kd, dt, overlap, s);
-    case kTma32x2: return dns_launch_tma<32, 2>(nf, maps[ia], maps[2], a, psi, b, ax, kd, dt, overlap, s);
-    case kTma64: return dns_launch_tma<64, 1>(nf, maps[ia], maps[2], a, psi, b, ax, kd, dt, overlap, s);
+    case kTma32: return dns_launch_tma<32, 1>(nf, maps[ia], maps[2], a, psi, b, ax, kd, dt, queue, overlap, s);
+    case kTma32x2: return dns_launch_tma<32, 2>(nf, maps[ia], maps[2], a, psi, b, ax, kd, dt, queue, overlap, s);
+    case kTma64: return dns_launch_tma<64, 1>(nf, maps[ia], maps[2], a, psi, b, ax, kd, dt, queue, overlap, s);
     case kTma32p:
-        return dns_launch_tma<32, 1, true>(nf, maps[ia], maps[2], a, psi, b, ax, kd, dt, overlap, s);
+        return dns_launch_tma<32, 1, true>(nf, maps[ia], maps[2], a, psi, b, ax, kd, dt, queue, overlap, s);
     }
     return cudaErrorInvalidValue;
 }
@@ -1269,6 +1272,11 @@ cudaError_t dns_run(int nf, float *u, float *u_tmp, const float *psi, double kap
                    : v == "t64" ? kTma64 : v == "t32p" ? kTma32p : kCp64;
     }
     if (!tma && g_dns_kind >= kTma32) g_dns_kind = kCp32;
+    DnsQueue queue;
+    if (nsteps > 0 && tma && (g_dns_kind < 0 || g_dns_kind >= kTma32)) {
+        const cudaError_t e = dns_queue(queue, s);
+        if (e != cudaSuccess) return e;
+    }
     if (g_dns_kind < 0 && nsteps > 0) {
         // one trial step of each into u_tmp (u is not modified), best of two
         cudaEvent_t e0, e1;
@@ -1280,7 +1288,7 @@ cudaError_t dns_run(int nf, float *u, float *u_tmp, const float *psi, double kap
             for (int rep = 0; rep < 3; ++rep) {
                 cudaEventRecord(e0, s);
                 cudaError_t e = dns_launch_kind(kind, nf, maps_of(kind), 0, u, psi, u_tmp, ax, kd,
-                                                (float)dt, false, s);
+                                                (float)dt, queue, false, s);
                 cudaEventRecord(e1, s);
                 if (e != cudaSuccess) return e;
                 cudaEventSynchronize(e1);
@@ -1299,7 +1307,7 @@ cudaError_t dns_run(int nf, float *u, float *u_tmp, const float *psi, double kap
     count_launches(nsteps);
     for (int st = 0; st < nsteps; ++st) {
         cudaError_t e = dns_launch_kind(g_dns_kind, nf, maps_of(g_dns_kind), ia, a, psi, b, ax, kd,
-                                        (float)dt, st > 0, s);
+                                        (float)dt, queue, st > 0, s);
         if (e != cudaSuccess) return e;
         float *t = a; a = b; b = t;
         ia ^= 1;

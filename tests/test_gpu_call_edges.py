@@ -113,3 +113,45 @@ def test_box_sums_of_unequal_nodes(mlsd, torch_mod, r, kind):
     V = V.cpu().numpy()
     assert V[0, 0] == 0.5 and np.all(np.abs(V.ravel()[1:] - mean) <=
                                      abs(mean) * 2.0**-24 * 1.01 + depth * 2.0**-53 * mag / (r * r) + 2.0**-150)
+
+
+def _dns(torch_mod, nf):
+    spec = flows.cellular_two_scale(1.0 / 3, 1.0 / 3, 5)
+    import paper_1510_00451_gb300 as m
+    psi = torch_mod.empty(nf, nf, dtype=torch_mod.float32, device="cuda:0")
+    m.grid_psi(spec, nf, psi)
+    h = 2 * np.pi / nf
+    u0 = torch_mod.tensor(flows.gaussian_u0(nf), dtype=torch_mod.float32, device="cuda:0")
+    return psi, u0, 0.2 * min(h * h / 4, h / 2)
+
+
+@pytest.mark.parametrize("pin,name", [("t32", "k_dns_tma<32,1>"), ("t32x2", "k_dns_tma<32,2>"),
+                                      ("t64", "k_dns_tma<64,1>"), ("t32p", "k_dns_tma<32,1,pairs>"),
+                                      ("32", "k_dns_step<32>")])
+@pytest.mark.parametrize("steps", [1, 4, 5])
+def test_captured_dns_replays(mlsd, torch_mod, monkeypatch, pin, name, steps):
+    # every replay of a captured run gives the direct run's bits, whatever ran before it
+    monkeypatch.setenv("MLSD_DNS_TY", pin)
+    nf = 512
+    psi, u0, dt = _dns(torch_mod, nf)
+    u, ut = u0.clone(), torch_mod.empty_like(u0)
+    v, vt = u0.clone(), torch_mod.empty_like(u0)
+    mlsd.dns_run(u, ut, psi, 0.02, dt, steps)
+    assert mlsd.dns_kernel() == name
+    ref = u.clone()
+    assert not torch_mod.equal(ref, u0)
+    g = torch_mod.cuda.CUDAGraph()
+    with torch_mod.cuda.graph(g):
+        mlsd.dns_run(u, ut, psi, 0.02, dt, steps)
+    mlsd.dns_run(v, vt, psi, 0.02, dt, 3)
+    for k in range(4):
+        u.copy_(u0)
+        ut.fill_(float("nan"))
+        g.replay()
+        assert torch_mod.equal(u, ref), k
+        if k == 2:
+            v.copy_(u0)
+            vt.fill_(float("nan"))
+            mlsd.dns_run(v, vt, psi, 0.02, dt, steps)
+            assert torch_mod.equal(v, ref)
+    assert mlsd.dns_status() == 0
