@@ -14,6 +14,7 @@
 // both RK stages fused per tile (u and psi staged with a halo of 2 in shared
 // memory), one pass over HBM per time step: read u, read psi, write u.
 #include <algorithm>
+#include <atomic>
 #include <cstdlib>
 #include <mutex>
 #include <string>
@@ -1194,10 +1195,10 @@ static cudaError_t dns_launch_tma(int nf, const CUtensorMap &ma, const CUtensorM
 // or 32 rows, 4 CTAs/SM), or persistent CTAs fed by tensor copies (32 rows with one or
 // two staging buffers, 64 rows with one; 32 rows with the f32x2 pair arithmetic).
 // Picked once per process by timing each on the caller's grid;
-// MLSD_DNS_TY = 64 | 32 | t32 | t32x2 | t64 | t32p pins one.
-static bool g_dns_multi = false;                 // the last run took several steps a launch
-enum DnsKind { kCp64, kCp32, kTma32, kTma32x2, kTma64, kTma32p, kDnsKinds };
-static int g_dns_kind = -1;
+// MLSD_DNS_TY = 64 | 32 | t32 | t32x2 | t64 | t32p pins one for the runs it is set for.
+enum DnsKind { kCp64, kCp32, kTma32, kTma32x2, kTma64, kTma32p, kSteps, kDnsKinds };
+static std::atomic<int> g_dns_choice{-1};        // the timed choice
+static std::atomic<int> g_dns_last{-1};          // the kernel of the last run
 
 static cudaError_t dns_launch_kind(int kind, int nf, const CUtensorMap *maps, int ia,
                                    const float *a, const float *psi, float *b, float ax, float kd,
@@ -1253,10 +1254,9 @@ cudaError_t dns_run(int nf, float *u, float *u_tmp, const float *psi, double kap
     const float ax = (float)(1.0 / (2.0 * h));
     const float kd = (float)(kappa / (h * h));
     if (nf <= kDnsMultiMax && !std::getenv("MLSD_DNS_TY")) {
-        g_dns_multi = true;
+        g_dns_last = kSteps;
         return dns_multi<false>(nf, u, u_tmp, psi, (float)dt * ax * ax, (float)dt * kd, nsteps, 0.f, 0.f, s);
     }
-    g_dns_multi = false;
     // tensor maps of u, u_tmp and psi; boxes of DLX x (DTY + 4), one map set per tile height
     CUtensorMap m32[3], m64[3];
     const bool tma = encode_f32_2d(&m32[0], u, nf, nf, DLX, 36) &&
@@ -1266,28 +1266,29 @@ cudaError_t dns_run(int nf, float *u, float *u_tmp, const float *psi, double kap
                      encode_f32_2d(&m64[1], u_tmp, nf, nf, DLX, 68) &&
                      encode_f32_2d(&m64[2], psi, nf, nf, DLX, 68);
     auto maps_of = [&](int kind) -> const CUtensorMap * { return kind == kTma64 ? m64 : m32; };
+    int kind = g_dns_choice;
     if (const char *env = std::getenv("MLSD_DNS_TY")) {
         const std::string v(env);
-        g_dns_kind = v == "32" ? kCp32 : v == "t32" ? kTma32 : v == "t32x2" ? kTma32x2
+        kind = v == "32" ? kCp32 : v == "t32" ? kTma32 : v == "t32x2" ? kTma32x2
                    : v == "t64" ? kTma64 : v == "t32p" ? kTma32p : kCp64;
     }
-    if (!tma && g_dns_kind >= kTma32) g_dns_kind = kCp32;
+    if (!tma && kind >= kTma32) kind = kCp32;
     DnsQueue queue;
-    if (nsteps > 0 && tma && (g_dns_kind < 0 || g_dns_kind >= kTma32)) {
+    if (nsteps > 0 && tma && (kind < 0 || kind >= kTma32)) {
         const cudaError_t e = dns_queue(queue, s);
         if (e != cudaSuccess) return e;
     }
-    if (g_dns_kind < 0 && nsteps > 0) {
+    if (kind < 0 && nsteps > 0) {
         // one trial step of each into u_tmp (u is not modified), best of two
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
         float best = 1e30f;
-        for (int kind = 0; kind < (tma ? (int)kDnsKinds : (int)kTma32); ++kind) {
+        for (int k = 0; k < (tma ? (int)kSteps : (int)kTma32); ++k) {
             float t = 1e30f;
             for (int rep = 0; rep < 3; ++rep) {
                 cudaEventRecord(e0, s);
-                cudaError_t e = dns_launch_kind(kind, nf, maps_of(kind), 0, u, psi, u_tmp, ax, kd,
+                cudaError_t e = dns_launch_kind(k, nf, maps_of(k), 0, u, psi, u_tmp, ax, kd,
                                                 (float)dt, queue, false, s);
                 cudaEventRecord(e1, s);
                 if (e != cudaSuccess) return e;
@@ -1297,16 +1298,18 @@ cudaError_t dns_run(int nf, float *u, float *u_tmp, const float *psi, double kap
                 if (rep > 0) t = std::min(t, ms);
             }
             count_launches(3);
-            if (t < best) { best = t; g_dns_kind = kind; }
+            if (t < best) { best = t; kind = k; }
         }
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
+        g_dns_choice = kind;
     }
+    g_dns_last = kind;
     float *a = u, *b = u_tmp;
     int ia = 0;
     count_launches(nsteps);
     for (int st = 0; st < nsteps; ++st) {
-        cudaError_t e = dns_launch_kind(g_dns_kind, nf, maps_of(g_dns_kind), ia, a, psi, b, ax, kd,
+        cudaError_t e = dns_launch_kind(kind, nf, maps_of(kind), ia, a, psi, b, ax, kd,
                                         (float)dt, queue, st > 0, s);
         if (e != cudaSuccess) return e;
         float *t = a; a = b; b = t;
@@ -1321,9 +1324,9 @@ const char *dns_kernel_name()
 {
     static const char *names[kDnsKinds] = {"k_dns_step<64>", "k_dns_step<32>", "k_dns_tma<32,1>",
                                            "k_dns_tma<32,2>", "k_dns_tma<64,1>",
-                                           "k_dns_tma<32,1,pairs>"};
-    if (g_dns_multi) return "k_dns_steps";
-    return g_dns_kind < 0 ? "" : names[g_dns_kind];
+                                           "k_dns_tma<32,1,pairs>", "k_dns_steps"};
+    const int kind = g_dns_last;
+    return kind < 0 ? "" : names[kind];
 }
 
 int dns_status_take(cudaStream_t s)

@@ -155,3 +155,19 @@ def test_captured_dns_replays(mlsd, torch_mod, monkeypatch, pin, name, steps):
             mlsd.dns_run(v, vt, psi, 0.02, dt, steps)
             assert torch_mod.equal(v, ref)
     assert mlsd.dns_status() == 0
+
+
+def test_pinned_dns_kernel_is_not_kept(mlsd, torch_mod, monkeypatch):
+    # a pin chooses the kernel of the runs it is set for; the timed choice stays
+    monkeypatch.delenv("MLSD_DNS_TY", raising=False)
+    psi, u, dt = _dns(torch_mod, 1152)
+    ut = torch_mod.empty_like(u)
+    mlsd.dns_run(u, ut, psi, 0.02, dt, 1)
+    chosen = mlsd.dns_kernel()
+    for pin, name in (("64", "k_dns_step<64>"), ("32", "k_dns_step<32>"), ("t32", "k_dns_tma<32,1>")):
+        monkeypatch.setenv("MLSD_DNS_TY", pin)
+        mlsd.dns_run(u, ut, psi, 0.02, dt, 1)
+        assert mlsd.dns_kernel() == name
+        monkeypatch.delenv("MLSD_DNS_TY")
+        mlsd.dns_run(u, ut, psi, 0.02, dt, 1)
+        assert mlsd.dns_kernel() == chosen
