@@ -1273,6 +1273,13 @@ cudaError_t dns_run(int nf, float *u, float *u_tmp, const float *psi, double kap
                    : v == "t64" ? kTma64 : v == "t32p" ? kTma32p : kCp64;
     }
     if (!tma && kind >= kTma32) kind = kCp32;
+    if (kind < 0) {
+        // nothing can be timed (nor the queue made) under capture: the per-tile kernel, for this run
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        const cudaError_t e = cudaStreamIsCapturing(s, &cs);
+        if (e != cudaSuccess) return e;
+        if (cs != cudaStreamCaptureStatusNone) kind = kCp32;
+    }
     DnsQueue queue;
     if (nsteps > 0 && tma && (kind < 0 || kind >= kTma32)) {
         const cudaError_t e = dns_queue(queue, s);

@@ -1,10 +1,13 @@
 """Calls at the edges of what the entry points accept."""
 import math
+import subprocess
+import sys
 
 import numpy as np
 import pytest
 
 from inputs import flows
+from tests.conftest import ROOT
 
 pytestmark = pytest.mark.gpu
 
@@ -171,3 +174,38 @@ def test_pinned_dns_kernel_is_not_kept(mlsd, torch_mod, monkeypatch):
         monkeypatch.delenv("MLSD_DNS_TY")
         mlsd.dns_run(u, ut, psi, 0.02, dt, 1)
         assert mlsd.dns_kernel() == chosen
+
+
+def test_first_large_dns_run_is_captured(torch_mod):
+    # a program that ran a small grid may capture its first large one: no kernel is timed under
+    # capture (a process of its own: the choice is made once per process)
+    code = """
+import numpy as np, torch
+import paper_1510_00451_gb300 as m
+from inputs import flows
+def case(nf):
+    psi = torch.empty(nf, nf, device='cuda:0')
+    m.grid_psi(flows.cellular_two_scale(1.0 / 3, 1.0 / 3, 5), nf, psi)
+    u0 = torch.tensor(flows.gaussian_u0(nf), dtype=torch.float32, device='cuda:0')
+    h = 2 * np.pi / nf
+    return psi, u0, torch.empty_like(u0), 0.2 * min(h * h / 4, h / 2)
+psi, u, ut, dt = case(256)
+m.dns_run(u, ut, psi, 0.02, dt, 3)
+psi, u0, ut, dt = case(1152)
+u = u0.clone()
+g = torch.cuda.CUDAGraph()
+torch.cuda.synchronize()
+with torch.cuda.graph(g):
+    m.dns_run(u, ut, psi, 0.02, dt, 3)
+assert torch.equal(u, u0)
+for k in range(2):
+    u.copy_(u0)
+    g.replay()
+    v = u0.clone()
+    m.dns_run(v, ut, psi, 0.02, dt, 3)
+    torch.cuda.synchronize()
+    assert float((u - v).abs().max()) <= 1e-6 and float((u - u0).abs().max()) > 1e-6
+print('captured')
+"""
+    out = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0 and "captured" in out.stdout, out.stderr[-2000:]
