@@ -432,7 +432,8 @@ int mlsd_check_wait_timeout(mlsd_levels *h, int which, void *cuda_stream);
  *   mass_out    host [nsteps + 1] or NULL: H^2 * sum(U) after each step (FP64);
  *               when non-NULL the call blocks until the steps are done.
  * Above 32^2 (FP64: 16^2) allocates, stream-ordered from the library's pool,
- * five N*N arrays (face coefficients and a field); and the mass list. */
+ * five N*N arrays (face coefficients and a field); with mass_out the list
+ * and, above those sizes, every tile's share of it (8 bytes a tile and step). */
 int mlsd_macro_step(int n_macro, void *U_dev, int precision, const double *K_dev, double dt,
                     int nsteps, double *mass_out_host, void *cuda_stream);
 

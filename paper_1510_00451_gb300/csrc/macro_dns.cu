@@ -1031,12 +1031,14 @@ static long long macro_mass_blocks(int N, int precision)
     return std::max(((long long)N * N + 255) / 256, macro_tiles(N, precision));
 }
 
-size_t macro_scratch_bytes(int N, int precision, int nsteps)
+// five fields, and with the mass record the tiles' shares of every step
+size_t macro_scratch_bytes(int N, int precision, int nsteps, bool mass)
 {
     const size_t rs = precision == MLSD_FP64 ? 8 : 4;
     const size_t NN = (size_t)N * N;
     if (macro_resident(N, precision)) return 0;
-    return 5 * NN * rs + 256 + (size_t)(nsteps + 1) * macro_mass_blocks(N, precision) * sizeof(double);
+    const size_t parts = mass ? ((size_t)nsteps + 1) * macro_mass_blocks(N, precision) : 0;
+    return 5 * NN * rs + 256 + parts * sizeof(double);
 }
 
 template <typename real, bool DIR>

@@ -176,7 +176,7 @@ cudaError_t dns_run_dirichlet(int nf, void *u, void *u_tmp, const float *psi, in
                               double kappa, double dt, int nsteps, double ul, double ur, void *scratch,
                               cudaStream_t s);
 size_t dns_dirichlet_scratch_bytes(int nf, int precision, int nsteps);
-size_t macro_scratch_bytes(int N, int precision, int nsteps);
+size_t macro_scratch_bytes(int N, int precision, int nsteps, bool mass);
 cudaError_t macro_dt_max(int N, const double *K, double *max_dev, cudaStream_t s);
 
 cudaError_t dns_run(int nf, float *u, float *u_tmp, const float *psi, double kappa, double dt,

@@ -1253,7 +1253,7 @@ int mlsd_macro_step(int n_macro, void *U_dev, int precision, const double *K_dev
     if (n_macro < 2 || !U_dev || !K_dev || !(dt > 0) || nsteps < 0) return MLSD_EINVAL;
     if (precision != MLSD_FP32 && precision != MLSD_FP64) return MLSD_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    const size_t sb = macro_scratch_bytes(n_macro, precision, nsteps);
+    const size_t sb = macro_scratch_bytes(n_macro, precision, nsteps, mass_out_host != nullptr);
     const size_t mb = mass_out_host ? (size_t)(nsteps + 1) * sizeof(double) : 0;
     void *scratch = nullptr;
     if (sb + mb) CK(ws_alloc(&scratch, sb + mb + 256, s));
@@ -1277,7 +1277,7 @@ int mlsd_macro_step_dirichlet(int n_macro, void *U_dev, int precision, const dou
     if (precision != MLSD_FP32 && precision != MLSD_FP64) return MLSD_EINVAL;
     if (!std::isfinite(u_left) || !std::isfinite(u_right)) return MLSD_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    const size_t sb = macro_scratch_bytes(n_macro, precision, nsteps);
+    const size_t sb = macro_scratch_bytes(n_macro, precision, nsteps, mass_out_host != nullptr);
     const size_t mb = mass_out_host ? (size_t)(nsteps + 1) * sizeof(double) : 0;
     void *scratch = nullptr;
     if (sb + mb) CK(ws_alloc(&scratch, sb + mb + 256, s));

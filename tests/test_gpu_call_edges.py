@@ -209,3 +209,19 @@ print('captured')
 """
     out = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert out.returncode == 0 and "captured" in out.stdout, out.stderr[-2000:]
+
+
+def test_macro_workspace_without_mass(mlsd, torch_mod):
+    # without the mass record the workspace does not grow with the number of steps: it would be
+    # 86 MB here.  The memory is the pool's until the next synchronisation, in pieces of 32 MB
+    N, steps = 33, 1200000
+    U = torch_mod.ones(N, N, dtype=torch_mod.float32, device="cuda:0")
+    K = torch_mod.ones(N * N, 3, dtype=torch_mod.float64, device="cuda:0")
+    mlsd.macro_step(U, K, 1e-4, 5, want_mass=False)
+    mlsd.Surrogate(1, 32, 8).close()                    # gives the pool's idle memory back
+    before = torch_mod.cuda.mem_get_info()[0]
+    mlsd.macro_step(U, K, 1e-4, steps, want_mass=False)
+    after = torch_mod.cuda.mem_get_info()[0]
+    torch_mod.cuda.synchronize()
+    assert before - after < 64 << 20
+    assert bool((U == 1.0).all())
