@@ -2,6 +2,7 @@
 // Algorithm 3 orchestration, error handling.
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -187,8 +188,10 @@ struct HostMode { int k1, k2; double re, im; };
 std::vector<HostMode> fold_modes(const std::vector<HostMode> &modes)
 {
     std::vector<HostMode> ms = modes;
-    for (HostMode &m : ms)
+    for (HostMode &m : ms) {
+        if (m.k1 == INT_MIN || m.k2 == INT_MIN) continue;      // no mirror among the ints: as it is
         if (m.k1 < 0 || (m.k1 == 0 && m.k2 < 0)) m = {-m.k1, -m.k2, m.re, -m.im};
+    }
     std::stable_sort(ms.begin(), ms.end(), [](const HostMode &a, const HostMode &b) {
         return a.k1 != b.k1 ? a.k1 < b.k1 : a.k2 < b.k2;
     });

@@ -225,3 +225,17 @@ def test_macro_workspace_without_mass(mlsd, torch_mod):
     torch_mod.cuda.synchronize()
     assert before - after < 64 << 20
     assert bool((U == 1.0).all())
+
+
+@pytest.mark.parametrize("k1,k2", [(-2**31, 3), (3, -2**31), (2**31 - 1, -5), (-2**31 + 1, 2), (0, -2**31)])
+def test_grid_psi_wave_numbers_of_any_int(mlsd, torch_mod, k1, k2):
+    # a point's phase is (k1 x + k2 y) mod nf: exact in integers, whatever the wave numbers
+    class Spec:
+        def as_arrays(self):
+            return (np.array([k1], np.int32), np.array([k2], np.int32), np.array([0.75]), np.array([-0.5]))
+    nf = 7
+    g = torch_mod.zeros(nf, nf, dtype=torch_mod.float32, device="cuda:0")
+    mlsd.grid_psi(Spec(), nf, g)
+    y, x = np.mgrid[:nf, :nf]
+    ph = 2 * np.pi * (((k1 % nf) * x + (k2 % nf) * y) % nf) / nf
+    assert np.abs(g.cpu().numpy() - (0.75 * np.cos(ph) + 0.5 * np.sin(ph))).max() < 4 * 2.0**-24
