@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(NT) k_macro_resident(int N, real *Ug, const do
             return k == 0 ? X[row[r + 1] + x] : k < 0 ? X[row[r + 1] + xw] : (east ? ur : X[row[r + 1] + xe]);
         }, d);
     };
-    for (int k = 1; k <= nsteps; ++k) {
+    for (int k = 0; k < nsteps; ++k) {
         if (own) {
             stage(U);
             s = held ? u : u + d[0];
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(NT) k_macro_resident(int N, real *Ug, const do
         }
         if (mass) {
             m = block_sum(m, red);
-            if (threadIdx.x == 0) mass[k] = m * H2;
+            if (threadIdx.x == 0) mass[k + 1LL] = m * H2;
         }
         __syncthreads();
     }
@@ -1059,7 +1059,7 @@ static cudaError_t macro_run_t(int N, real *U, const double *K, double dt, int n
     }
     real *co = static_cast<real *>(scratch), *V = co + 4 * (size_t)NN;
     constexpr int S = F64 ? kSteps64 : kSteps32, TY = F64 ? kTileY64 : kTileY32;
-    const int launches = (nsteps + S - 1) / S;
+    const int launches = nsteps / S + (nsteps % S ? 1 : 0);
     // the tile launches ping-pong between U and V and end in U
     const bool start_in_V = launches & 1;
     count_launches(1);
@@ -1072,17 +1072,17 @@ static cudaError_t macro_run_t(int N, real *U, const double *K, double dt, int n
     count_launches(launches + (mass ? 3 : 0));
     if (mass) k_mass_part<real><<<nb, th, 0, s>>>(NN, U, part);
     real *a = start_in_V ? V : U, *b = start_in_V ? U : V;
-    for (int k = 0; k < nsteps; k += S) {
+    for (long long k = 0; k < nsteps; k += S) {
         const cudaError_t e = launch_chained(
             k_macro_tile<real, kTileX, TY, S, DIR>, grid, (T::NT + 31) / 32 * 32, 0, k > 0, s, N, a, b, co,
-            std::min(S, nsteps - k), mass ? part + stride + (size_t)k * tiles : nullptr, r);
+            (int)std::min<long long>(S, nsteps - k), mass ? part + stride + (size_t)k * tiles : nullptr, r);
         if (e != cudaSuccess) return e;
         std::swap(a, b);
     }
     if (mass) {
         k_mass_final<<<1, 128, 0, s>>>(1, nb, part, H * H, mass);
         if (nsteps > 0)
-            k_mass_final<<<(nsteps + 127) / 128, 128, 0, s>>>(nsteps, (int)tiles, part + stride, H * H, mass + 1);
+            k_mass_final<<<(unsigned)((nsteps + 127LL) / 128), 128, 0, s>>>(nsteps, (int)tiles, part + stride, H * H, mass + 1);
     }
     return cudaGetLastError();
 }
@@ -1226,7 +1226,7 @@ static cudaError_t dns_multi(int nf, float *u, float *u_tmp, const float *psi, f
     constexpr int EX = 64, EY = 40, S = 4, R = 4;
     using D = DnsSteps<EX, EY, S, R>;
     // an even number of launches, the steps spread evenly over them (one step: a copy back)
-    int launches = (nsteps + S - 1) / S;
+    int launches = nsteps / S + (nsteps % S ? 1 : 0);
     if ((launches & 1) && nsteps > 1) ++launches;
     const dim3 grid((unsigned)((nf + D::TX - 1) / D::TX), (unsigned)((nf + D::TY - 1) / D::TY));
     count_launches(launches);
