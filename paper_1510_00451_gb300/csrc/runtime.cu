@@ -535,6 +535,12 @@ int build(const mlsd_problem *p, cudaStream_t s, mlsd_levels *h)
 // Autotuner: time every compiled tiling of the patch kernel on a sample of the
 // level's patches (short fixed window, the level's own band, base kappa I) and
 // keep the fastest per (device, n, precision) for the rest of the process.
+// At that base B12 = 0, and the one-CTA kernels leave the cross term out, which levels above a
+// chain's finest do not.  The picks hold for those all the same: of 8192 fields of 32^2, 888
+// steps, with the term, 4x8 takes 6.53 ms, packed 4x4 7.46, row-paired 4x8 7.43; of 2048 fields
+// of 64^2 4x8 6.65, 4x8m3 7.30, 4x8m2r 7.55; 4x4 is the FP64 pick with and without it.  A trial
+// with B12 != 0 picked packed 4x4 for 32^2, by the set-up's share of its 64 steps (0.604 ms against
+// 0.605), and a chain of three such levels took 20.4 ms instead of 18.6.
 std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int>, std::pair<int, int>> g_tune;   // -> (bx, code(by, minb, packed))
 
