@@ -1387,16 +1387,20 @@ cudaError_t dns_run_dirichlet(int nf, void *u, void *u_tmp, const float *psi, in
     count_launches((aE ? 1 : 0) + (long long)nsteps);
     if (aE) k_dns_dir_coef<<<(unsigned)((n2 + 255) / 256), 256, 0, s>>>(nf, psi, r2 * cA, r2 * cD, aE, aN);
     // tiles of 32 rows where they give every SM one, else of 8 (an SM's FP64 rate decides)
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
     const unsigned gx = (unsigned)((nf + kD64TX - 1) / kD64TX);
-    const bool tall = (long long)gx * ((nf + 31) / 32) >= 152;
+    const bool tall = (long long)gx * ((nf + 31) / 32) >= sms;
     const int ty = tall ? 32 : 8, nt = 32 * (ty + 4) / kD64R;
     const dim3 grid(gx, (unsigned)((nf + ty - 1) / ty));
     const auto fn = tall ? k_dns_dir_step64<32> : k_dns_dir_step64<8>;
     const double sq2 = 1.4142135623730951;
     double *a = static_cast<double *>(u), *b = static_cast<double *>(u_tmp);
     for (int k = 0; k < nsteps; ++k) {
-        const cudaError_t e = launch_chained(fn, grid, nt, 0, k > 0, s, nf, a, b, aE, aN, psi, r2 * cA,
-                                             r2 * cD, ul, ur, sq2 * ul, sq2 * ur);
+        e = launch_chained(fn, grid, nt, 0, k > 0, s, nf, a, b, aE, aN, psi, r2 * cA, r2 * cD, ul, ur, sq2 * ul,
+                           sq2 * ur);
         if (e != cudaSuccess) return e;
         std::swap(a, b);
     }
