@@ -33,7 +33,8 @@ struct PatchParams {
     const int *pidx;         // patch index of work-item pair (item >> 1), or nullptr: identity
     long long tile = 0;      // 0: band is the level grid; else per-patch tiles, patch p at band + p * tile
     const int *count_dev = nullptr;   // if set: only the first 2 * (*count_dev) items, taken by a
-                                      // grid-stride loop (a launch sized before the count is known)
+                                      // grid-stride loop (a launch sized before the count is known);
+                                      // FP32 kernels only
 };
 
 

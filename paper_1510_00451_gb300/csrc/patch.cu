@@ -60,6 +60,8 @@ int patch_variants(int n, int precision, std::vector<PatchVariant> &out)
 cudaError_t launch_patch(const PatchVariant &v, const PatchParams &p, long long grid,
                          cudaStream_t s)
 {
+    // k_patch_solve64 takes one item per CTA (surrogate levels, whose counts are on the device, are FP32)
+    if (p.count_dev && v.precision == MLSD_FP64) return cudaErrorNotSupported;
     cudaError_t e = cudaFuncSetAttribute(v.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)v.smem);
     if (e != cudaSuccess) return e;
