@@ -211,7 +211,7 @@ cudaError_t sur_grad(int h, int M, const void *X, const float *Y, const float *w
 struct SurTc {
     int max_rows = 0, ldT = 0;
     __nv_bfloat16 *XT = nullptr;          // [640][ldT]
-    __nv_bfloat16 *AT[3] = {};            // [h][ldT] transposed activations
+    __nv_bfloat16 *AT[2] = {};            // [h][ldT] transposed activations (dW4 reads the third untransposed)
     __nv_bfloat16 *WT[2] = {};            // [h][h] transposed W_1, W_2
     __nv_bfloat16 *dZ[2] = {};            // [max_rows][h] bfloat16 gradients
     __nv_bfloat16 *dZT[3] = {};           // [h][ldT], per hidden layer

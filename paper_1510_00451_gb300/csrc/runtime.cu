@@ -1546,7 +1546,7 @@ int mlsd_surrogate_create(int members, int hidden, int max_batch, mlsd_surrogate
         const size_t T = (size_t)t.ldT;
         void *p = nullptr;
         if (!rc) { rc = sur_alloc(s, &p, (size_t)MLSD_SUR_IN * T * 2); t.XT = (__nv_bfloat16 *)p; }
-        for (int l = 0; l < 3 && !rc; ++l) { rc = sur_alloc(s, &p, H * T * 2); t.AT[l] = (__nv_bfloat16 *)p; }
+        for (int l = 0; l < 2 && !rc; ++l) { rc = sur_alloc(s, &p, H * T * 2); t.AT[l] = (__nv_bfloat16 *)p; }
         for (int l = 0; l < 2 && !rc; ++l) { rc = sur_alloc(s, &p, H * H * 2); t.WT[l] = (__nv_bfloat16 *)p; }
         for (int l = 0; l < 2 && !rc; ++l) { rc = sur_alloc(s, &p, M * H * 2); t.dZ[l] = (__nv_bfloat16 *)p; }
         for (int l = 0; l < 3 && !rc; ++l) { rc = sur_alloc(s, &p, H * T * 2); t.dZT[l] = (__nv_bfloat16 *)p; }

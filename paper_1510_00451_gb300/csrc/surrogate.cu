@@ -1197,7 +1197,7 @@ __global__ void __launch_bounds__(256) k_out_bwd(OutBwd a)
 // slices' partials added in order, four entries a thread.  Blocks of their biases: db_l[r] = the
 // sum of row r of dZ_l^T (bfloat16, row stride ld a multiple of 8, zero padding), one warp a
 // row, each lane 16-byte vectors 8 k apart, then the warp tree.  Then the output layer's (dW4 and
-// db4 from k_out_bwd_w's chunks in order), and the loss, its blocks' shares added in FP64.
+// db4 from k_out_bwd's chunks in order), and the loss, its blocks' shares added in FP64.
 struct GradReduce {
     const float *part[3];
     float *w[3], *b[3];
@@ -1434,7 +1434,7 @@ cudaError_t sur_grad_tc(int h, int M, const void *X, const float *Y, const float
     const __nv_bfloat16 *in = static_cast<const __nv_bfloat16 *>(X);
     for (int l = 0; l < 3 && e == cudaSuccess; ++l) {
         e = gemm_tc(0, M, h, L.din[l], in, L.din[l], wb + L.w[l], L.din[l], wf + L.b[l], Z[l],
-                    nullptr, Aact[l], tc.AT[l], ldT, status, l > 0, s);
+                    nullptr, Aact[l], l < 2 ? tc.AT[l] : nullptr, ldT, status, l > 0, s);
         in = static_cast<const __nv_bfloat16 *>(Aact[l]);
     }
     if (e != cudaSuccess) return e;
