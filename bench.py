@@ -39,13 +39,26 @@ UNIT = "cell-updates/s"
 # Algorithmic FP32 work of k_patch_solve.  Per cell-update (one cell of one field,
 # one full Heun step): stage 1 = 4 FADD + 6 FFMA, stage 2 = 4 FADD + 7 FFMA.
 # Per cell-update inside the averaging window, add the flux sums: 2 FFMA + 1 FADD.
-# On the finest level (B12 = 0) the kernels leave out the cross term: one FADD and one
-# FFMA less per stage.
+# On the finest level (B12 = 0) the one-CTA kernels with their coefficients in registers
+# (_leaves_out_cross) leave out the cross term: one FADD and one FFMA less per stage.
 OPS_PER_CELL_UPDATE = 21       # FP32-pipe instructions
 OPS_PER_WINDOW_UPDATE = 3
 FLOP_PER_CELL_UPDATE = 34
 FLOP_PER_WINDOW_UPDATE = 5
 OPS_CROSS, FLOP_CROSS = 4, 6
+
+
+def _leaves_out_cross(info, size=None):
+    """Whether the kernel of a level description leaves out the cross term where B12 = 0.  Of a
+    level's classes the description shows the tiling of the one with the most work: for the others
+    (size given) the tuner's usual picks, one CTA at 32^2 and 64^2, clusters or tensor memory above."""
+    if info["level_launch"]:
+        return False
+    if size is not None and size != info["n"]:
+        return size <= 64
+    return info["cluster"] == 1 and info["split"] == 0 and info["coef_tmem"] == 0
+
+
 # DRAM bytes (read + write) per patch-solve launch of this workload, measured by ncu
 # (dram__bytes_read.sum + dram__bytes_write.sum) on the three level launches of
 # `--case profile`: the same grids, bands and tiling as the timed step (the window
@@ -723,19 +736,23 @@ def uneven_case(n_avg=256):
     sm_count = torch.cuda.get_device_properties(dev).multi_processor_count
     issue_peak = sm_count * 128 * peaks.get("sm_max_mhz", 2070.0) * 1e6
     per_level = []
+    tiles = [lv.info(l + 1) for l in range(L)]
     for l in range(L):
         cls = lv.profile_collect_classes(l + 1)
         ms = sum(v[0] for v in cls.values())
         n = sum(v[1] for v in cls.values())
         cu_l, _, wu_l = work[l]
-        per_cell = OPS_PER_CELL_UPDATE - (OPS_CROSS if l == L - 1 else 0)
-        ops = cu_l * per_cell + wu_l * OPS_PER_WINDOW_UPDATE
+        # fixed window without burn-in: every step of every field is inside it
+        cu_of = {size: count * 2 * size * size * n_avg for size, count in hist[l].items()}
+        no_cross = {s for s in cu_of if l == L - 1 and _leaves_out_cross(tiles[l], s)}
+        cross_cu = sum(cu_of[s] for s in no_cross)
+        ops = cu_l * OPS_PER_CELL_UPDATE - cross_cu * OPS_CROSS + wu_l * OPS_PER_WINDOW_UPDATE
         classes = []
         for size, (ms_c, n_c) in sorted(cls.items()):
             if size == 0 or ms_c <= 0:
                 continue
-            # fixed window without burn-in: every step of every field is inside it
-            cu_c = hist[l][size] * 2 * size * size * n_avg
+            cu_c = cu_of[size]
+            per_cell = OPS_PER_CELL_UPDATE - (OPS_CROSS if size in no_cross else 0)
             classes.append({"n": size, "patches": hist[l][size], "kernel_ms": ms_c,
                             "cell_updates_per_s": cu_c / (ms_c * 1e-3),
                             "fp32_issue_frac": cu_c * (per_cell + OPS_PER_WINDOW_UPDATE)
@@ -745,9 +762,8 @@ def uneven_case(n_avg=256):
                           "cell_updates_per_s": cu_l / (ms * 1e-3) if ms > 0 else None,
                           "fp32_issue_frac": ops / (ms * 1e-3) / issue_peak if ms > 0 else None,
                           "classes": classes})
-    tiles = [lv.info(l + 1) for l in range(L)]
     ops = sum(w[0] * OPS_PER_CELL_UPDATE + w[2] * OPS_PER_WINDOW_UPDATE for w in work)
-    ops -= work[-1][0] * OPS_CROSS
+    ops -= cross_cu * OPS_CROSS                   # of the last level, the finest
     return {"workload": "continuous spectrum |k|<=256, 8 octave levels, 65536 patches/level, "
                         f"sizes 32^2..256^2 by the size rule, {n_avg}-step window",
             "cell_updates_per_s": cu / t, "seconds": t, "cell_updates": cu,
@@ -826,8 +842,8 @@ def mlp_case(M=65536, members=4, hidden=256):
 
 def series_case(N=256, reps=3):
     """Surrogate features of every patch of the 6th-octave level (65536 patches of
-    32^2): k_features (DFT window) and k_series (moments T_2..T_19 by FFTs and
-    their resummation), timed with CUDA events (ncu case)."""
+    32^2): k_series (the low-mode window, moments T_2..T_19 by FFTs and their
+    resummation), timed with CUDA events (ncu case)."""
     import torch
     import inputs
     import paper_1510_00451_gb300 as mlsd
@@ -1082,9 +1098,10 @@ def main():
                           "cell_updates": cu_l, "max_steps_per_patch": work[l][1],
                           "cell_updates_per_s": cu_l / (ms / args.steps * 1e-3) if ms > 0 else None,
                           "k_eff_tensors_per_s": N * N / (ms / args.steps * 1e-3) if ms > 0 else None})
-    kern_ops = args.steps * (cell_updates * OPS_PER_CELL_UPDATE - work[-1][0] * OPS_CROSS
+    cross_cu = work[-1][0] if _leaves_out_cross(lv.info(L)) else 0
+    kern_ops = args.steps * (cell_updates * OPS_PER_CELL_UPDATE - cross_cu * OPS_CROSS
                              + window_updates * OPS_PER_WINDOW_UPDATE)
-    kern_flop = args.steps * (cell_updates * FLOP_PER_CELL_UPDATE - work[-1][0] * FLOP_CROSS
+    kern_flop = args.steps * (cell_updates * FLOP_PER_CELL_UPDATE - cross_cu * FLOP_CROSS
                               + window_updates * FLOP_PER_WINDOW_UPDATE)
     assert lv.status() == 0
     ms_step = ranks_max(ms_step, world, dev)
@@ -1187,7 +1204,8 @@ def main():
                      "kernel": "k_patch_solve", "launches": kern_n,
                      "kernel_ms_per_step": kern_ms / args.steps,
                      "algorithmic": f"{OPS_PER_CELL_UPDATE} FP32 FADD/FMUL/FFMA per cell-update "
-                                    f"({OPS_PER_CELL_UPDATE - OPS_CROSS} on the finest level) "
+                                    f"({OPS_PER_CELL_UPDATE - (OPS_CROSS if cross_cu else 0)} on the "
+                                    f"finest level) "
                                     f"+ {OPS_PER_WINDOW_UPDATE} per averaging-window cell-update",
                      "window_fraction": window_updates / cell_updates,
                      "peak_basis": f"{sm_count} SMs x 128 FP32 lanes x {sm_max:.0f} MHz, one "

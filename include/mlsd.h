@@ -433,7 +433,9 @@ int mlsd_check_wait_timeout(mlsd_levels *h, int which, void *cuda_stream);
  *               when non-NULL the call blocks until the steps are done.
  * Above 32^2 (FP64: 16^2) allocates, stream-ordered from the library's pool,
  * five N*N arrays (face coefficients and a field); with mass_out the list
- * and, above those sizes, every tile's share of it (8 bytes a tile and step). */
+ * and, above those sizes, every tile's share of it (8 bytes a tile and step).
+ * Under capture the workspace is a memory node of the graph, which then takes
+ * one instantiation at a time.                                              */
 int mlsd_macro_step(int n_macro, void *U_dev, int precision, const double *K_dev, double dt,
                     int nsteps, double *mass_out_host, void *cuda_stream);
 
@@ -491,8 +493,10 @@ const char *mlsd_dns_kernel(void);
  * periodic in x2), posed on [0, 2 pi] x [0, 2 pi) as mlsd_macro_step_dirichlet:
  * column 0 of u_dev is set to u_left and held, the virtual column nf has the
  * value u_right; psi (and so v) stays periodic.  FP32: four steps per launch;
- * FP64: a step per launch, from face coefficients formed once per run in a
- * stream-ordered scratch of 2 nf^2 doubles; any nf >= 4.
+ * FP64: a step per launch, up to 8192^2 from face coefficients formed once per run
+ * in a stream-ordered scratch of 2 nf^2 doubles (under capture a memory node of the
+ * graph, which then takes one instantiation at a time); above, or where the scratch
+ * finds no memory, formed in every step, with the same results.  Any nf >= 4.
  *   u_dev, u_tmp_dev  device [nf][nf], float (MLSD_FP32) or double (MLSD_FP64);
  *                     u_tmp_dev is a caller-provided work field
  *   psi_dev           device [nf][nf] float (mlsd_grid_psi)

@@ -365,7 +365,7 @@ def dns_status(stream=None):
 
 
 def dns_kernel():
-    """Name of the DNS kernel this process picked ("" before the first run)."""
+    """Name of the DNS kernel of the last dns_run ("" before the first run)."""
     return _lib.mlsd_dns_kernel().decode()
 
 

@@ -11,8 +11,10 @@
 // The mass H^2 sum(U) of every step is summed in FP64.
 //
 // DNS: u_t = v1 D0x u + v2 D0y u + kappa (Dxx + Dyy) u, v = (-D0y psi, D0x psi),
-// both RK stages fused per tile (u and psi staged with a halo of 2 in shared
-// memory), one pass over HBM per time step: read u, read psi, write u.
+// both RK stages fused per tile.  Large periodic grids: u and psi staged with a halo of 2
+// in shared memory, one pass over HBM per time step (read u, read psi, write u).  Grids up to
+// 1024^2, and Dirichlet in x1 in FP32: four steps of a tile with its halo per launch.  Dirichlet in
+// FP64: a step per launch, from coefficients formed once per run.
 #include <algorithm>
 #include <atomic>
 #include <cstdlib>
@@ -907,8 +909,8 @@ __global__ void k_dns_vmax(int nf, const float *psi, float ax, unsigned *out)
 // each becomes its 24-bit significand in units of 2^(E - 150 - shift), so that n of them fit
 // 62 bits.  That is exact where every node but zeros is within 2^shift (2^26 at least) of the
 // largest, and the sum is rounded once to FP64.  Nodes further apart, which integers would round to
-// their unit, are added in FP64, as infinities and NaN are.  The 8 warps' FP64 work is left to one of them (a warp
-// with one box takes as long as one with 8).  8192^2 onto 64^2, 128^2, 512^2: 288, 367, 2081 us
+// their unit, are added in FP64, as infinities and NaN are.  The 8 warps' FP64 work is left to one
+// of them (a warp with one box takes as long as one with 8).  8192^2 onto 64^2, 128^2, 512^2: 288, 367, 2081 us
 // for a CTA a box in FP64; 130, 136, 150 so (118, 122, 144 without looking for nodes too far
 // apart, each of them then off by up to 2^-50 of the largest); 311, 314, 359 where every box has such
 // nodes (reading them once: 40).  What bounds it: the integer operations, about 27 a node.
